@@ -87,7 +87,7 @@ struct Carve {
 struct ScratchOffsets {
   uint64_t slot_of, expert_of, last_use, clock, stats, tr_n, tr_expert, tr_slot, tr_hit;
   uint64_t zpart, idx, g, uniq, uslot, umiss, asg_off, asg, pos_slot, info, miss_list, h, part;
-  uint64_t work, err, tb_off, sx, sb, sy, sidx, sw, stage;
+  uint64_t work, err, tb_off, sx, sb, sy, sidx, sw, stage, xs, hs, xe;
   uint64_t total;
 };
 
@@ -115,7 +115,7 @@ ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   o.pos_slot = c.take<int32_t>((uint64_t)Tm * k);
   o.info = c.take<int32_t>(2 + E);
   o.miss_list = c.take<int32_t>(E + S);
-  o.h = c.take<float>((uint64_t)Tm * k * I);
+  o.h = c.take<float>(k * I);
   o.part = c.take<float>(Tm > 1 ? (uint64_t)Tm * k * H : 1);
   o.work = c.take<uint64_t>(16);  // the fused FFN's grid arrival counter, alone on its 128-byte line
   o.err = c.take<unsigned>(1);
@@ -127,6 +127,9 @@ ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   o.sw = c.take<float>((uint64_t)Tm * k);
   // calls with several waves stage the next wave's misses: one payload per slot (T_max > 1)
   o.stage = c.take<uint8_t>(Tm > 1 ? (uint64_t)S * make_layout(m).stride : 0);
+  o.xs = c.take<uint8_t>(Tm > 1 ? stream_bytes(Tm, (int)H) : 0);
+  o.hs = c.take<uint8_t>(Tm > 1 ? stream_bytes(Tm * (int)k, (int)I) : 0);
+  o.xe = c.take<int32_t>(Tm);
   o.total = c.off;
   return o;
 }
@@ -359,6 +362,9 @@ int create_ctx(mf_ctx_t** out, const mf_model_t* m, const mf_plan_t* p, int devi
   d.work = reinterpret_cast<unsigned long long*>(base + so.work);
   d.stage = Tm > 1 ? base + so.stage : nullptr;
   d.err = reinterpret_cast<unsigned*>(base + so.err);
+  d.xs = base + so.xs;
+  d.hs = base + so.hs;
+  d.xe = reinterpret_cast<int32_t*>(base + so.xe);
   d.tb_off = reinterpret_cast<int32_t*>(base + so.tb_off);
   c->stage_x = reinterpret_cast<float*>(base + so.sx);
   c->stage_bias = reinterpret_cast<float*>(base + so.sb);
@@ -400,6 +406,10 @@ int create_ctx(mf_ctx_t** out, const mf_model_t* m, const mf_plan_t* p, int devi
   }
   c->decode_pipe = decode_pipe_ok(d) && getenv("MF_DECODE_SIMPLE") == nullptr;
   c->ffn_fused = c->decode_pipe && ffn_fused_ok(d) && getenv("MF_DECODE_UNFUSED") == nullptr;
+  if (Tm > 1 && stream_tensor_maps(c)) {
+    free_ctx(c);
+    return MF_E_CUDA;
+  }
   c->tmaps_ok = prefill_shape_ok(d.H, d.I) && prefill_tensor_maps(c) == 0;
   c->prefill_min_t = 0;
   if (c->tmaps_ok && gemm_at_create(*m, Tm)) {
@@ -561,23 +571,32 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
     long long width = accesses_max - (long long)w * S;
     return (int)(width > S ? S : width);
   };
-  MF_CUDA(cudaEventRecord(c->ev_fork[0], s));
-  MF_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork[0], 0));
-  if (c->file) MF_CUDA(enqueue_file_reads(c, layer, 0, false, c->side));  // wave 0's misses, file -> staging
-  timer_mark(c, kTMaterialize, 0, c->side);
-  MF_CUDA(launch_materialize(d, layer, 0, wave_width(0), c->side, nullptr, gemm));
-  timer_mark(c, kTMaterialize, 1, c->side);
-  MF_CUDA(cudaEventRecord(c->ev_join[0], c->side));
-  if (gemm) MF_CUDA(launch_tile_x(d, x, T, s));  // the GEMM's x tiles, while wave 0 materialises
+  // A call of one wave below the GEMM threshold has nothing to overlap with the copy: it stays on `s`
+  // (a fork and join through events costs several microseconds of idle GPU).
+  const bool inline_mat = n_waves == 1 && !gemm;
+  cudaStream_t ms = inline_mat ? s : c->side;
+  if (!inline_mat) {
+    MF_CUDA(cudaEventRecord(c->ev_fork[0], s));
+    MF_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork[0], 0));
+  }
+  if (c->file) MF_CUDA(enqueue_file_reads(c, layer, 0, false, ms));  // wave 0's misses, file -> staging
+  timer_mark(c, kTMaterialize, 0, ms);
+  MF_CUDA(launch_materialize(d, layer, 0, wave_width(0), ms, nullptr, T > 1 && !inline_mat));
+  timer_mark(c, kTMaterialize, 1, ms);
+  if (!inline_mat) MF_CUDA(cudaEventRecord(c->ev_join[0], c->side));
+  // the activations in the form the expert kernels read, while wave 0 materialises
+  if (gemm)
+    MF_CUDA(launch_tile_x(d, x, T, s));
+  else if (T > 1)
+    MF_CUDA(launch_split_x(d, x, T, s));
   auto stage_next = [&](int w) -> cudaError_t {  // side stream: wave w's misses into the stage
     timer_mark(c, kTMaterialize, 0, c->side);
-    cudaError_t e = launch_materialize(d, layer, w, wave_width(w), c->side, d.stage, gemm);
+    cudaError_t e = launch_materialize(d, layer, w, wave_width(w), c->side, d.stage, true);
     timer_mark(c, kTMaterialize, 1, c->side);
     return e;
   };
   if (staged) MF_CUDA(stage_next(1));
   for (int w = 0; w < n_waves; ++w) {
-    const int width = wave_width(w);
     if (w > 0) {  // side stream, once wave w - 1 has computed: wave w's misses into their slots
       MF_CUDA(cudaEventRecord(c->ev_fork[w], s));
       MF_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork[w], 0));
@@ -586,13 +605,13 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
       } else {
         if (c->file) MF_CUDA(enqueue_file_reads(c, layer, w, false, c->side));
         timer_mark(c, kTMaterialize, 0, c->side);
-        MF_CUDA(launch_materialize(d, layer, w, width, c->side, nullptr, gemm));
+        MF_CUDA(launch_materialize(d, layer, w, wave_width(w), c->side, nullptr, true));
         timer_mark(c, kTMaterialize, 1, c->side);
       }
       MF_CUDA(cudaEventRecord(c->ev_join[w], c->side));
       if (staged && w + 1 < n_waves) MF_CUDA(stage_next(w + 1));  // overlaps wave w's compute
     }
-    MF_CUDA(cudaStreamWaitEvent(s, c->ev_join[w], 0));  // wave w's experts are in their slots
+    if (!inline_mat) MF_CUDA(cudaStreamWaitEvent(s, c->ev_join[w], 0));  // wave w's experts are in their slots
     if (gemm) {
       timer_mark(c, kTPrefill, 0, s);
       MF_CUDA(launch_prefill_gateup(d, c->tm_gu, layer, w, s));
@@ -609,8 +628,10 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
     timer_mark(c, kTGateUp, 0, s);
     if (pipe)
       MF_CUDA(launch_gateup_single(d, layer, x, s));
+    else if (T == 1)
+      MF_CUDA(launch_gateup(d, layer, x, s));
     else
-      MF_CUDA(launch_gateup(d, layer, w, (int)width, x, s));
+      MF_CUDA(launch_stream_gateup(d, c->ts_gu, layer, w, T, s));
     timer_mark(c, kTGateUp, 1, s);
     timer_mark(c, kTDown, 0, s);
     if (pipe)
@@ -618,7 +639,7 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
     else if (T == 1)
       MF_CUDA(launch_down_single(d, layer, y, s));
     else
-      MF_CUDA(launch_down_partial(d, layer, w, (int)width, s));
+      MF_CUDA(launch_stream_down(d, c->ts_d, layer, w, T, s));
     if (T > 1 && w == n_waves - 1) MF_CUDA(launch_combine(d, T, y, s));
     timer_mark(c, kTDown, 1, s);
   }

@@ -69,7 +69,12 @@ struct Dev {
   int32_t* pos_slot;   // [T_max * k]   slot serving assignment t * k + j
   int32_t* info;       // [2 + E]       U, number of waves, misses of wave w at 2 + w
   int32_t* miss_list;  // [E + S_alloc] unique index of miss m of wave w at w * S_active + m
-  float* h;            // [T_max * k][I]  SwiGLU activations
+  float* h;            // [k][I]  SwiGLU activations (T = 1)
+  // T > 1 below the GEMM threshold: activations as three exact bf16 pieces, per K chunk of 128 one run of
+  // kStreamChunkBytes = [piece][128], in the streaming kernels' K order
+  uint8_t* xs;         // [T_max][ceil(H / 128)]      x
+  uint8_t* hs;         // [T_max * k][ceil(I / 128)]  SwiGLU activations
+  int32_t* xe;         // [T_max]  exponent by which each token's x was scaled
   float* part;         // [T_max * k][H]  per-assignment down outputs (T > 1)
   int32_t* tb_off;     // [E + 1]       128-assignment blocks before unique expert u (T > 1)
   // tensor-core path (many tokens per expert): operand tiles in the MMA's shared-memory order,
@@ -247,6 +252,8 @@ struct mf_ctx {
   int prefill_min_t;  // calls with T >= this use the tensor-core grouped GEMMs (0 = never)
   uint8_t* gemm_scratch;  // x and h tiles of the tensor-core path (allocated when first enabled)
   bool tmaps_ok;
+  CUtensorMap ts_gu[2], ts_d[2];  // the same regions for the streaming kernels: [0] boxes of 64 rows' codes
+                                  // of 128 weights, [1] boxes of 64 rows' 8 scales
   CUtensorMap tm_gu[2], tm_d[2];  // the slot pool's gate/up and down row records as 3-D byte tensors:
                                   // [0] boxes of one step's codes, [1] boxes of one scale group
 };
@@ -272,9 +279,9 @@ cudaError_t launch_materialize(const Dev& d, int layer, int wave, int max_miss, 
                                uint8_t* dst_stage = nullptr, bool spread = false);
 // the wave's staged payloads into their slots
 cudaError_t launch_stage_commit(const Dev& d, int layer, int wave, const uint8_t* stage, cudaStream_t s);
-cudaError_t launch_gateup(const Dev& d, int layer, int wave, int wave_width, const float* x, cudaStream_t s);
+// one token, one warp per weight row (shapes the pipelined kernels do not take)
+cudaError_t launch_gateup(const Dev& d, int layer, const float* x, cudaStream_t s);
 cudaError_t launch_down_single(const Dev& d, int layer, float* y, cudaStream_t s);
-cudaError_t launch_down_partial(const Dev& d, int layer, int wave, int wave_width, cudaStream_t s);
 cudaError_t launch_combine(const Dev& d, int T, float* y, cudaStream_t s);
 cudaError_t launch_reset(const Dev& d, cudaStream_t s);
 // batch-1 decode: pipelined gate/up + SwiGLU and down + combine (shared-memory bulk-copy stages)
@@ -285,12 +292,24 @@ bool decode_pipe_ok(const Dev& d);
 // both projections of one token in one cooperative launch (d.work holds its arrival counter)
 bool ffn_fused_ok(const Dev& d);
 cudaError_t launch_ffn_single(const Dev& d, int layer, const float* x, float* y, cudaStream_t s);
+// a few to a few hundred tokens: each wave's experts streamed through the warp-level MMA (mf_stream.cu)
+constexpr int kStreamCols = 32;          // assignments per work unit
+constexpr int kStreamChunkBytes = 768;   // one assignment's activation pieces of 128 values
+size_t stream_bytes(int n, int K);       // bytes of n assignments' pieces of K values
+int stream_tensor_maps(mf_ctx* c);       // encode ts_gu / ts_d for the context's pool; 0 on success
+cudaError_t launch_split_x(const Dev& d, const float* x, int T, cudaStream_t s);
+cudaError_t launch_stream_gateup(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s);
+cudaError_t launch_stream_down(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s);
 // many tokens per expert: tcgen05 grouped GEMMs (gate/up + SwiGLU, down) per wave
 constexpr int kPrefillMinTokens = 256;
 bool prefill_shape_ok(int hidden, int inter);
 uint64_t prefill_tiles_max(int T, int k, int E);  // bound on the 128-assignment blocks of a call
 uint64_t prefill_scratch_bytes(int T_max, int k, int E, int hidden, int inter);
 int prefill_tensor_maps(mf_ctx* c);  // encode tm_gu / tm_d for the context's pool; 0 on success
+// one region of every slot as a 3-D byte tensor (byte in row record, row, slot plane): boxes of box_bytes x
+// box_rows, swizzled by `swizzle` bytes (0, 64 or 128); 0 on success
+int encode_slot_region(CUtensorMap* tm, void* base, uint64_t rec_bytes, uint64_t rows, uint64_t planes,
+                       uint64_t plane_stride, uint32_t box_bytes, uint32_t box_rows, int swizzle);
 cudaError_t launch_tile_x(const Dev& d, const float* x, int T, cudaStream_t s);
 cudaError_t launch_prefill_gateup(const Dev& d, const CUtensorMap* tm, int layer, int wave, cudaStream_t s);
 cudaError_t launch_prefill_down(const Dev& d, const CUtensorMap* tm, int layer, int wave, cudaStream_t s);

@@ -117,7 +117,7 @@ extern "C" int mf_expert_ffn_noalloc(const mf_model_t* model, const void* expert
     if (launch_gateup_single(d, 0, x, s) != cudaSuccess) return MF_E_CUDA;
     if (launch_down_single_pipe(d, 0, y, s) != cudaSuccess) return MF_E_CUDA;
   } else {
-    if (launch_gateup(d, 0, 0, m.top_k, x, s) != cudaSuccess) return MF_E_CUDA;
+    if (launch_gateup(d, 0, x, s) != cudaSuccess) return MF_E_CUDA;
     if (launch_down_single(d, 0, y, s) != cudaSuccess) return MF_E_CUDA;
   }
   return MF_OK;

@@ -558,24 +558,6 @@ cudaError_t launch_k(const Dev& d, const CUtensorMap* tm, int layer, int wave, c
   return cudaGetLastError();
 }
 
-using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// One region of every slot as a 3-D byte tensor: (byte in row record, row, slot plane).
-int encode_region(EncodeTiled enc, CUtensorMap* tm, void* base, uint64_t rec_bytes, uint64_t rows, uint64_t planes,
-                  uint64_t plane_stride, uint32_t box_bytes) {
-  const cuuint64_t dims[3] = {rec_bytes, rows, planes};
-  const cuuint64_t strides[2] = {rec_bytes, plane_stride};
-  const cuuint32_t box[3] = {box_bytes, (cuuint32_t)kBM, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-                 CUDA_SUCCESS
-             ? 0
-             : -1;
-}
-
 }  // namespace
 
 // shapes the GEMM path serves: whole 128-row blocks in both projections (which also makes the
@@ -592,20 +574,38 @@ uint64_t prefill_scratch_bytes(int T_max, int k, int E, int H, int I) {
   return prefill_tiles_max(T_max, k, E) * (uint64_t)kBN * (uint64_t)(H + I) * 4;  // hi + lo bf16
 }
 
-int prefill_tensor_maps(mf_ctx* c) {
+int encode_slot_region(CUtensorMap* tm, void* base, uint64_t rec_bytes, uint64_t rows, uint64_t planes,
+                       uint64_t plane_stride, uint32_t box_bytes, uint32_t box_rows, int swizzle) {
+  using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q;
   if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
       q != cudaDriverEntryPointSuccess || !fn)
     return -1;
-  const EncodeTiled enc = reinterpret_cast<EncodeTiled>(fn);
+  const cuuint64_t dims[3] = {rec_bytes, rows, planes};
+  const cuuint64_t strides[2] = {rec_bytes, plane_stride};
+  const cuuint32_t box[3] = {box_bytes, box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUtensorMapSwizzle sw = swizzle == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+                                : swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                : CU_TENSOR_MAP_SWIZZLE_NONE;
+  return reinterpret_cast<EncodeTiled>(fn)(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, dims, strides, box, estr,
+                                           CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? 0
+             : -1;
+}
+
+int prefill_tensor_maps(mf_ctx* c) {
   const Dev& d = c->d;
   const uint32_t cb = d.qtype == MF_Q8_0 ? 32 : 16;
   const uint64_t planes = (uint64_t)d.L * d.S_alloc;
   for (int m = 0; m < 2; ++m) {  // code boxes (one step), scale boxes (one group)
     const uint32_t box = m ? kScaleBox : cb;
-    if (encode_region(enc, &c->tm_gu[m], d.pool, d.lay.rs_gu, (uint64_t)d.I, planes, d.lay.stride, box)) return -1;
-    if (encode_region(enc, &c->tm_d[m], d.pool + d.lay.d_off, d.lay.rs_d, (uint64_t)d.H, planes, d.lay.stride, box))
+    if (encode_slot_region(&c->tm_gu[m], d.pool, d.lay.rs_gu, (uint64_t)d.I, planes, d.lay.stride, box, kBM, 0)) return -1;
+    if (encode_slot_region(&c->tm_d[m], d.pool + d.lay.d_off, d.lay.rs_d, (uint64_t)d.H, planes, d.lay.stride, box, kBM, 0))
       return -1;
   }
   return 0;

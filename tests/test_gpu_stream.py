@@ -1,0 +1,40 @@
+"""Calls of 2 to 255 tokens (the streaming expert kernels) at the edges of their tiles, against the
+CPU oracle: rows and K lengths that are not multiples of the 64-record boxes or the 128-weight
+stages, and experts that serve 1, 8, 9, 32, 33 or more assignments."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from mfharness import Ctx, Payloads, Shape, assert_outputs_close
+
+pytestmark = pytest.mark.gpu
+
+# The kernels keep 24 bits of every operand and sum in fp32: a few roundings of 2^-24 on each of the
+# three products of a layer, grown by the sums' lengths (square root of 500 terms at most here), stay
+# below 1e-6 of the row in the 2-norm.
+REL = 1e-6
+
+
+@pytest.mark.parametrize("qtype", [synth.Q8_0, synth.Q4_0])
+@pytest.mark.parametrize("H,I", [(32, 32), (160, 96), (416, 352), (512, 640)])
+def test_stream_tile_edges(qtype, H, I):
+    E, k = 12, 3
+    shape = Shape(1, H, E, k, I, qtype, model_seed=7)
+    ctx = Ctx(shape, E, max_tokens=70)
+    pays = Payloads(shape)
+    try:
+        for T in (2, 8, 9, 32, 33, 70):
+            x = synth.activations(T, 0, 0, 0, T, H)
+            # expert 0 serves every token, expert 1 all but one, the third choice is spread out
+            sets = np.stack([np.zeros(T, int), np.where(np.arange(T) == 1, 2, 1), 3 + np.arange(T) % (E - 3)], 1)
+            bias = synth.plant_bias(sets.astype(np.int32), E)
+            y, idx, _ = ctx.forward(0, x, bias, T)
+            yo, io, _ = oracle.layer(pays.for_layer(0, range(E)), qtype, H, I, k, ctx.wr_host[0], bias, x)
+            assert np.array_equal(idx, io)
+            assert_outputs_close(y, yo, f"T {T}")
+            rel = np.linalg.norm(y - yo, axis=1) / np.linalg.norm(yo, axis=1)
+            assert rel.max() <= REL, (T, rel.max())
+        assert ctx.mf.mf_check(ctx.h) == 0
+    finally:
+        ctx.close()
