@@ -542,13 +542,12 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
   timer_mark(c, kTRouter, 0, s);
   MF_CUDA(launch_router(d, x, router_w, logit_bias, T, layer, s));
   timer_mark(c, kTRouter, 1, s);
+  const bool gemm = T > 1 && c->prefill_min_t > 0 && T >= c->prefill_min_t;
   if (T > 1) {  // one token per call: the router's last block resolved the slots already
     timer_mark(c, kTResolve, 0, s);
-    MF_CUDA(launch_resolve(d, layer, T, s));
+    MF_CUDA(launch_resolve(d, layer, T, x, !gemm, s));
     timer_mark(c, kTResolve, 1, s);
   }
-
-  const bool gemm = T > 1 && c->prefill_min_t > 0 && T >= c->prefill_min_t;
 
   if (T == 1 && c->ffn_fused) {  // one launch: expert FFN, with the misses materialised inside
     if (c->file) MF_CUDA(enqueue_file_reads(c, layer, 0, true, s));  // the misses, file -> staging
@@ -581,17 +580,13 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
   }
   if (c->file) MF_CUDA(enqueue_file_reads(c, layer, 0, false, ms));  // wave 0's misses, file -> staging
   timer_mark(c, kTMaterialize, 0, ms);
-  MF_CUDA(launch_materialize(d, layer, 0, wave_width(0), ms, nullptr, T > 1 && !inline_mat));
+  MF_CUDA(launch_materialize(d, layer, 0, wave_width(0), ms, nullptr, T > 1 && !inline_mat, inline_mat && !c->file));
   timer_mark(c, kTMaterialize, 1, ms);
   if (!inline_mat) MF_CUDA(cudaEventRecord(c->ev_join[0], c->side));
-  // the activations in the form the expert kernels read, while wave 0 materialises
-  if (gemm)
-    MF_CUDA(launch_tile_x(d, x, T, s));
-  else if (T > 1)
-    MF_CUDA(launch_split_x(d, x, T, s));
+  if (gemm) MF_CUDA(launch_tile_x(d, x, T, s));  // the GEMM's x tiles, while wave 0 materialises
   auto stage_next = [&](int w) -> cudaError_t {  // side stream: wave w's misses into the stage
     timer_mark(c, kTMaterialize, 0, c->side);
-    cudaError_t e = launch_materialize(d, layer, w, wave_width(w), c->side, d.stage, true);
+    cudaError_t e = launch_materialize(d, layer, w, wave_width(w), c->side, d.stage, true, false);
     timer_mark(c, kTMaterialize, 1, c->side);
     return e;
   };
@@ -605,7 +600,7 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
       } else {
         if (c->file) MF_CUDA(enqueue_file_reads(c, layer, w, false, c->side));
         timer_mark(c, kTMaterialize, 0, c->side);
-        MF_CUDA(launch_materialize(d, layer, w, wave_width(w), c->side, nullptr, true));
+        MF_CUDA(launch_materialize(d, layer, w, wave_width(w), c->side, nullptr, true, false));
         timer_mark(c, kTMaterialize, 1, c->side);
       }
       MF_CUDA(cudaEventRecord(c->ev_join[w], c->side));
@@ -631,7 +626,7 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
     else if (T == 1)
       MF_CUDA(launch_gateup(d, layer, x, s));
     else
-      MF_CUDA(launch_stream_gateup(d, c->ts_gu, layer, w, T, s));
+      MF_CUDA(launch_stream_gateup(d, c->ts_gu, layer, w, T, inline_mat, s));
     timer_mark(c, kTGateUp, 1, s);
     timer_mark(c, kTDown, 0, s);
     if (pipe)

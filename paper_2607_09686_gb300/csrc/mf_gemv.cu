@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(256) k_down_single(Dev d, int layer, float* __
 
 // y[t][c] = sum_j g[t,j] part[t*k+j][c], j in rank order
 __global__ void k_combine(Dev d, int T, float* __restrict__ y) {
+  pdl_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)T * d.H) return;
   const int t = (int)(i / d.H), c = (int)(i % d.H);
@@ -190,8 +191,7 @@ cudaError_t launch_down_single(const Dev& d, int layer, float* y, cudaStream_t s
 cudaError_t launch_combine(const Dev& d, int T, float* y, cudaStream_t s) {
   const size_t n = (size_t)T * d.H;
   same_carveout(k_combine);
-  k_combine<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, T, y);
-  return cudaGetLastError();
+  return launch_pdl(true, k_combine, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, d, T, y);
 }
 
 }  // namespace mf

@@ -165,6 +165,30 @@ __device__ __forceinline__ bool counter_wait(const unsigned long long* cnt, unsi
 // pdl_trigger: allow the dependent launch to be scheduled (its blocks start as SMs free up).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A launch whose blocks may be scheduled while the stream's previous kernel ends (every kernel launched
+// this way calls pdl_wait before it touches global memory); a plain launch where that is refused or not
+// asked for (overlap false: after an event wait the predecessor is not a kernel of this stream).
+template <class... P, class... A>
+cudaError_t launch_pdl(bool overlap, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (overlap) {
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    if (e == cudaSuccess) return e;
+    cudaGetLastError();
+  }
+  cfg.numAttrs = 0;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
 // bulk copy global -> this CTA's shared memory, completing `bytes` on the mbarrier
 // (addresses 16-byte aligned, bytes a multiple of 16)
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -272,11 +296,13 @@ constexpr int kTiledMinT = 16;
 size_t router_part_pairs(int T_max, int E, int H);
 cudaError_t launch_router(const Dev& d, const float* x, const float* wr, const float* bias, int T, int layer,
                           cudaStream_t s, float* x_copy = nullptr);
-cudaError_t launch_resolve(const Dev& d, int layer, int T, cudaStream_t s);
+// with `split`, the same launch also writes the call's activation pieces (d.xs, d.xe) from x
+cudaError_t launch_resolve(const Dev& d, int layer, int T, const float* x, bool split, cudaStream_t s);
 // dst_stage null: each miss into its slot; else miss m of the wave to dst_stage + m * stride.
-// spread: one small block per SM (beside the persistent GEMM kernels), else a few large blocks
+// spread: one small block per SM (beside the persistent expert kernels), else a few large blocks.
+// overlap: launched programmatically (launch_pdl)
 cudaError_t launch_materialize(const Dev& d, int layer, int wave, int max_miss, cudaStream_t s,
-                               uint8_t* dst_stage = nullptr, bool spread = false);
+                               uint8_t* dst_stage, bool spread, bool overlap);
 // the wave's staged payloads into their slots
 cudaError_t launch_stage_commit(const Dev& d, int layer, int wave, const uint8_t* stage, cudaStream_t s);
 // one token, one warp per weight row (shapes the pipelined kernels do not take)
@@ -297,8 +323,8 @@ constexpr int kStreamCols = 32;          // assignments per work unit
 constexpr int kStreamChunkBytes = 768;   // one assignment's activation pieces of 128 values
 size_t stream_bytes(int n, int K);       // bytes of n assignments' pieces of K values
 int stream_tensor_maps(mf_ctx* c);       // encode ts_gu / ts_d for the context's pool; 0 on success
-cudaError_t launch_split_x(const Dev& d, const float* x, int T, cudaStream_t s);
-cudaError_t launch_stream_gateup(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s);
+cudaError_t launch_stream_gateup(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, bool overlap,
+                                 cudaStream_t s);
 cudaError_t launch_stream_down(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s);
 // many tokens per expert: tcgen05 grouped GEMMs (gate/up + SwiGLU, down) per wave
 constexpr int kPrefillMinTokens = 256;

@@ -33,6 +33,8 @@ constexpr int kMatThreadsDense = 512;  // one block per 8 SMs
 // dst_stage: null to write each miss into its slot, else miss m of the wave goes to
 // dst_stage + m * stride
 __global__ void __launch_bounds__(kMatThreadsDense) k_materialize(Dev d, int layer, int wave, uint8_t* dst_stage) {
+  pdl_trigger();
+  pdl_wait();
   const int n_miss = d.info[2 + wave];
   const size_t nvec = d.lay.stride / 16;  // 16-byte vectors per payload
   const size_t step = (size_t)gridDim.x * blockDim.x * kUnroll;
@@ -110,15 +112,13 @@ cudaError_t max_shared_carveout() {
 }
 
 cudaError_t launch_materialize(const Dev& d, int layer, int wave, int max_miss, cudaStream_t s, uint8_t* dst_stage,
-                               bool spread) {
+                               bool spread, bool overlap) {
   if (max_miss <= 0) return cudaSuccess;
   cudaError_t e = max_shared_carveout();
   if (e != cudaSuccess) return e;
   if (spread)
-    k_materialize<<<n_sm(), kMatThreadsSpread, 0, s>>>(d, layer, wave, dst_stage);
-  else
-    k_materialize<<<(n_sm() + 7) / 8, kMatThreadsDense, 0, s>>>(d, layer, wave, dst_stage);
-  return cudaGetLastError();
+    return launch_pdl(overlap, k_materialize, dim3(n_sm()), dim3(kMatThreadsSpread), 0, s, d, layer, wave, dst_stage);
+  return launch_pdl(overlap, k_materialize, dim3((n_sm() + 7) / 8), dim3(kMatThreadsDense), 0, s, d, layer, wave, dst_stage);
 }
 
 cudaError_t launch_stage_commit(const Dev& d, int layer, int wave, const uint8_t* stage, cudaStream_t s) {

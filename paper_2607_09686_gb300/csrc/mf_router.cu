@@ -116,6 +116,47 @@ __device__ __forceinline__ bool cluster_rank_zero() {
   return r == 0;
 }
 
+// Rank by counting: position of expert e = experts with a larger logit, or equal and lower id; the k
+// first to s_sel / s_zsel.  tpe consecutive lanes share an expert, each counting over every tpe-th other
+// expert.  The block's z and s_sel are written before (with a barrier); ends with a barrier.
+template <int kThreads>
+__device__ __forceinline__ void rank_topk(const float* s_z, int E, int k, int* s_sel, float* s_zsel) {
+  const int tid = threadIdx.x;
+  int tpe = 1;
+  while (tpe < 32 && tpe * 2 * E <= kThreads) tpe *= 2;
+  const int per_pass = kThreads / tpe, part = tid % tpe;
+  for (int e0 = 0; e0 < E; e0 += per_pass) {  // block-uniform
+    const int e = e0 + tid / tpe;
+    const bool valid = e < E;
+    const float z = valid ? s_z[e] : 0.f;
+    int r = 0;
+    if (valid)
+      for (int e2 = part; e2 < E; e2 += tpe) {
+        const float z2 = s_z[e2];
+        r += (z2 > z) || (z2 == z && e2 < e);
+      }
+    for (int off = tpe >> 1; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    if (valid && part == 0 && r < k) {
+      s_sel[r] = e;
+      s_zsel[r] = z;
+    }
+  }
+  __syncthreads();
+}
+
+// softmax over the chosen, by one warp: lane j < k holds exp(z_j - z_0); fixed shuffle-tree sum
+__device__ __forceinline__ void softmax_topk(const Dev& d, int t, int k, const int* s_sel, const float* s_zsel) {
+  const int lane = threadIdx.x & 31;
+  const float ex = lane < k ? expf(s_zsel[lane] - s_zsel[0]) : 0.f;
+  float den = ex;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+  if (lane < k) {
+    d.idx[(size_t)t * k + lane] = s_sel[lane];
+    d.g[(size_t)t * k + lane] = ex / den;
+  }
+}
+
 __global__ void __launch_bounds__(kThreadsR)
     k_router(Dev d, const float* __restrict__ x, const float* __restrict__ wr, const float* __restrict__ bias, int T,
              int layer, int fuse_resolve, float* __restrict__ x_copy, int nc) {
@@ -213,43 +254,10 @@ __global__ void __launch_bounds__(kThreadsR)
   if (rank != 0) return;
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-  // rank by counting: position of expert e = experts with a larger logit, or equal and lower id
-  // (s_sel starts as 0..k-1: a valid choice even where the logits are not ordered, e.g. NaN).
-  // tpe consecutive lanes share an expert, each counting over every tpe-th other expert.
-  if (tid < k) s_sel[tid] = tid;
+  if (tid < k) s_sel[tid] = tid;  // a valid choice even where the logits are not ordered (NaN)
   __syncthreads();
-  {
-    int tpe = 1;
-    while (tpe < 32 && tpe * 2 * E <= kThreadsR) tpe *= 2;
-    const int per_pass = kThreadsR / tpe, part = tid % tpe;
-    for (int e0 = 0; e0 < E; e0 += per_pass) {  // block-uniform
-      const int e = e0 + tid / tpe;
-      const bool valid = e < E;
-      const float z = valid ? s_z[e] : 0.f;
-      int r = 0;
-      if (valid)
-        for (int e2 = part; e2 < E; e2 += tpe) {
-          const float z2 = s_z[e2];
-          r += (z2 > z) || (z2 == z && e2 < e);
-        }
-      for (int off = tpe >> 1; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
-      if (valid && part == 0 && r < k) {
-        s_sel[r] = e;
-        s_zsel[r] = z;
-      }
-    }
-  }
-  __syncthreads();
-  if (warp == 0) {  // softmax over the chosen: lane j < k holds exp(z_j - z_0); fixed shuffle-tree sum
-    const float ex = lane < k ? expf(s_zsel[lane] - s_zsel[0]) : 0.f;
-    float den = ex;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
-    if (lane < k) {
-      d.idx[(size_t)t * k + lane] = s_sel[lane];
-      d.g[(size_t)t * k + lane] = ex / den;
-    }
-  }
+  rank_topk<kThreadsR>(s_z, E, k, s_sel, s_zsel);
+  if (warp == 0) softmax_topk(d, t, k, s_sel, s_zsel);
   if (!resolve) return;
 
   // One token per call: the k chosen experts are distinct, so the accesses are the chosen
@@ -282,7 +290,7 @@ __global__ void __launch_bounds__(kThreadsR)
 // and experts tx + 16j (j < 4).  Columns are taken two at a time with f32x2 arithmetic (the same
 // IEEE operations as dot2, on two lanes): each output keeps one compensated pair for its even
 // and one for its odd columns, added error-free at the end.  The pairs of every K split go to
-// scratch; k_topk_tiled (one warp per token) adds them in split order, rounds once, adds the
+// scratch; k_topk_tiled (one block per token) adds them, rounds once, adds the
 // bias, ranks and takes the softmax exactly as the one-token path does.
 constexpr int kTT = 32, kTE = 64, kHC = 32, kThreadsT = 256;
 constexpr int kPadT = kHC + 4;  // shared row stride in floats: 16 rows read together hit 2 bank phases
@@ -355,6 +363,8 @@ __global__ void __launch_bounds__(kThreadsT)
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  pdl_trigger();
+  pdl_wait();
   uint64_t S[2][4], C[2][4];  // [token][expert]: (even-column, odd-column) pairs
 #pragma unroll
   for (int a = 0; a < 2; ++a)
@@ -402,52 +412,54 @@ __global__ void __launch_bounds__(kThreadsT)
   }
 }
 
-constexpr int kTokW = 8;  // tokens (warps) per block of k_topk_tiled
+constexpr int kThreadsTop = 256;
 
-__global__ void __launch_bounds__(kTokW * 32)
+// One block per token: the K splits' pairs of an expert are added by P threads (P a power of two, as
+// many as fit; each adds every P-th split in order, eight loads in flight, then thread 0 the P partial
+// pairs in order), the rest as in k_router.  (One warp per token with one load in flight at a time took
+// 87 us for the 44 splits of 64 tokens at hidden 2816 and 31 us for 4096 tokens.)
+__global__ void __launch_bounds__(kThreadsTop)
     k_topk_tiled(Dev d, const float2* __restrict__ part, const float* __restrict__ bias, int T, int ks) {
-  extern __shared__ __align__(16) float s_zt[];  // [kTokW][E]
-  __shared__ int s_sel[kTokW][kMaxTopK];
-  __shared__ float s_zs[kTokW][kMaxTopK];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = (int)blockIdx.x * kTokW + warp;
-  if (t >= T) return;  // warp-uniform; no block-wide barrier below
-  const int E = d.E, k = d.k;
-  float* z = s_zt + (size_t)warp * E;
-  for (int e = lane; e < E; e += 32) {
-    float2 p = part[(size_t)t * E + e];
-    for (int sp = 1; sp < ks; ++sp) {
-      const float2 q = part[((size_t)sp * T + t) * E + e];
-      pair_add(p.x, p.y, q.x, q.y);
-    }
-    float v = __fadd_rn(p.x, p.y);
-    if (bias) v = __fadd_rn(v, bias[(size_t)t * E + e]);
-    z[e] = v;
-  }
-  __syncwarp();
-  if (lane < k) s_sel[warp][lane] = lane;  // valid even where the logits are not ordered (NaN)
-  __syncwarp();
-  for (int e = lane; e < E; e += 32) {  // rank by counting, ties to the lower id
-    const float v = z[e];
-    int r = 0;
-    for (int e2 = 0; e2 < E; ++e2) {
-      const float v2 = z[e2];
-      r += (v2 > v) || (v2 == v && e2 < e);
-    }
-    if (r < k) {
-      s_sel[warp][r] = e;
-      s_zs[warp][r] = v;
-    }
-  }
-  __syncwarp();
-  const float ex = lane < k ? expf(s_zs[warp][lane] - s_zs[warp][0]) : 0.f;
-  float den = ex;
+  __shared__ float s_z[kMaxExperts];
+  __shared__ float2 s_p[kThreadsTop];
+  __shared__ int s_sel[kMaxTopK];
+  __shared__ float s_zs[kMaxTopK];
+  const int tid = threadIdx.x, t = blockIdx.x, E = d.E, k = d.k;
+  int P = 1;
+  while (P * 2 <= ks && P * 2 * E <= kThreadsTop) P *= 2;
+  const int per = kThreadsTop / P, p = tid / per;
+  pdl_trigger();
+  pdl_wait();
+  if (tid < k) s_sel[tid] = tid;  // valid even where the logits are not ordered (NaN)
+  for (int e0 = 0; e0 < E; e0 += per) {  // block-uniform
+    const int e = e0 + tid % per;
+    float2 a = make_float2(0.f, 0.f);
+    if (e < E) {
+      for (int s0 = p; s0 < ks; s0 += 8 * P) {
+        float2 q[8];
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
-  if (lane < k) {
-    d.idx[(size_t)t * k + lane] = s_sel[warp][lane];
-    d.g[(size_t)t * k + lane] = ex / den;
+        for (int u = 0; u < 8; ++u)
+          if (s0 + u * P < ks) q[u] = part[((size_t)(s0 + u * P) * T + t) * E + e];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (s0 + u * P < ks) pair_add(a.x, a.y, q[u].x, q[u].y);
+      }
+    }
+    s_p[tid] = a;
+    __syncthreads();
+    if (p == 0 && e < E) {
+      for (int i = 1; i < P; ++i) {
+        const float2 q = s_p[tid + i * per];
+        pair_add(a.x, a.y, q.x, q.y);
+      }
+      float v = __fadd_rn(a.x, a.y);
+      if (bias) v = __fadd_rn(v, bias[(size_t)t * E + e]);
+      s_z[e] = v;
+    }
+    __syncthreads();
   }
+  rank_topk<kThreadsTop>(s_z, E, k, s_sel, s_zs);
+  if (tid < 32) softmax_topk(d, t, k, s_sel, s_zs);
 }
 
 // K splits for T tokens: about kTiledBlocks blocks when the tiles alone are fewer.  A constant
@@ -467,17 +479,10 @@ cudaError_t launch_router_tiled(const Dev& d, const float* x, const float* wr, c
                                 cudaStream_t s) {
   const int ks = tiled_splits(T, d.E, d.H);
   const int nch = d.H / kHC, cps = (nch + ks - 1) / ks;
-  k_logits_tiled<<<dim3((d.E + kTE - 1) / kTE, (T + kTT - 1) / kTT, ks), kThreadsT, 0, s>>>(x, wr, T, d.E, d.H, cps,
-                                                                                            d.zpart);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_pdl(true, k_logits_tiled, dim3((d.E + kTE - 1) / kTE, (T + kTT - 1) / kTT, ks),
+                                   dim3(kThreadsT), 0, s, x, wr, T, d.E, d.H, cps, d.zpart);
   if (e != cudaSuccess) return e;
-  const size_t smem = (size_t)kTokW * d.E * sizeof(float);
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_topk_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  k_topk_tiled<<<(T + kTokW - 1) / kTokW, kTokW * 32, smem, s>>>(d, d.zpart, bias, T, ks);
-  return cudaGetLastError();
+  return launch_pdl(true, k_topk_tiled, dim3(T), dim3(kThreadsTop), 0, s, d, (const float2*)d.zpart, bias, T, ks);
 }
 
 }  // namespace

@@ -34,7 +34,7 @@
 // assignments of an expert); above about 16 assignments per expert the MMA (m16n8k16 runs at 2 cycles
 // per SM).  The codes stay in registers between the conversion and the MMA, and the unit's rows are the
 // MMA's M side, so a lightly loaded expert wastes only MMA columns, of which there are 8.
-#include "mf_dequant.cuh"
+#include "mf_stream.cuh"
 
 namespace mf {
 namespace {
@@ -43,7 +43,7 @@ using dq::kQ4;
 using dq::kQ8;
 
 constexpr int kRecs = 64;                       // row records per box
-constexpr int kKC = 128;                        // weights of K per stage
+constexpr int kKC = kStreamK;                   // weights of K per stage
 constexpr int kSeg = 4;                         // stages whose blocks are summed before they join the row's sum
 constexpr int kSCols = kStreamCols;             // assignments per unit
 constexpr int kSWarps = 16;                     // consumer warps
@@ -138,24 +138,6 @@ __device__ __forceinline__ void load_a(const unsigned char* lo, const unsigned c
     codes_q4(v & 0x0F0F0F0Fu, a[0][1], a[0][3]);
     codes_q4((v >> 4) & 0x0F0F0F0Fu, a[1][1], a[1][3]);
   }
-}
-
-// position of element e (of a 32-weight block) in the activation pieces
-template <int QT>
-__device__ __forceinline__ int stream_pos(int e) {
-  if constexpr (QT == kQ8) return e;
-  return ((e & 12) << 1) | ((e & 16) >> 2) | (e & 3);
-}
-
-// v = p0 + p1 + p2 exactly, each a bfloat16 (the top 8 bits of v, of the remainder, and the last 8)
-__device__ __forceinline__ void split3(float v, uint16_t (&p)[3]) {
-  const uint32_t b0 = __float_as_uint(v) & 0xFFFF0000u;
-  const float r1 = v - __uint_as_float(b0);
-  const uint32_t b1 = __float_as_uint(r1) & 0xFFFF0000u;
-  const float r2 = r1 - __uint_as_float(b1);
-  p[0] = (uint16_t)(b0 >> 16);
-  p[1] = (uint16_t)(b1 >> 16);
-  p[2] = (uint16_t)(__float_as_uint(r2) >> 16);
 }
 
 struct SUnit {
@@ -418,43 +400,6 @@ __global__ void __launch_bounds__(kSThreads, 1)
   __syncthreads();
 }
 
-// x [T][H] -> the pieces of 2^-e x, [T][ceil(H / 128)][3][128] in the consumers' K order, and e [T]
-template <int QT>
-__global__ void __launch_bounds__(256) k_split_x(Dev d, const float* __restrict__ x) {
-  __shared__ float s_m[8];
-  pdl_wait();
-  const int H = d.H, KC = (H + kKC - 1) / kKC;
-  const float4* row = reinterpret_cast<const float4*>(x + (size_t)blockIdx.x * H);
-  uint8_t* out = d.xs + (size_t)blockIdx.x * KC * kColBytes;
-  float m = 0.f;
-  for (int i = threadIdx.x; i < H / 4; i += 256) {
-    const float4 v = row[i];
-    m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = m;
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 8; ++i) m = fmaxf(m, s_m[i]);
-  const int e = dq::vec_exponent(m);
-  if (threadIdx.x == 0) d.xe[blockIdx.x] = e;
-  for (int i = threadIdx.x; i < H / 4; i += 256) {  // four values in a row stay together in the pieces
-    const float4 f = row[i];
-    const float v[4] = {f.x, f.y, f.z, f.w};
-    uint16_t p[4][3];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) split3(dq::scale2(v[q], -e), p[q]);
-    const int el = 4 * i;
-    uint16_t* o = reinterpret_cast<uint16_t*>(out + (size_t)(el / kKC) * kColBytes) +
-                  ((el & (kKC - 1) & ~31) | stream_pos<QT>(el & 31));
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      *reinterpret_cast<uint2*>(o + c * kKC) =
-          make_uint2(p[0][c] | (uint32_t)p[1][c] << 16, p[2][c] | (uint32_t)p[3][c] << 16);
-  }
-}
-
 int sm_count_s() {
   static int n = 0;
   if (!n) {
@@ -467,12 +412,12 @@ int sm_count_s() {
 }
 
 template <int QT, int NT>
-cudaError_t launch_s(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s) {
+cudaError_t launch_s(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, bool overlap,
+                     cudaStream_t s) {
   const StreamCfg f = stream_cfg(d, T);
   cudaError_t e = cudaFuncSetAttribute(k_stream<QT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.total);
   if (e != cudaSuccess) return e;
-  k_stream<QT, NT><<<sm_count_s(), kSThreads, f.total, s>>>(tm[0], tm[1], d, layer, wave, f);
-  return cudaGetLastError();
+  return launch_pdl(overlap, k_stream<QT, NT>, dim3(sm_count_s()), dim3(kSThreads), f.total, s, tm[0], tm[1], d, layer, wave, f);
 }
 
 }  // namespace
@@ -493,20 +438,15 @@ int stream_tensor_maps(mf_ctx* c) {
   return 0;
 }
 
-cudaError_t launch_split_x(const Dev& d, const float* x, int T, cudaStream_t s) {
-  if (d.qtype == MF_Q8_0)
-    k_split_x<kQ8><<<T, 256, 0, s>>>(d, x);
-  else
-    k_split_x<kQ4><<<T, 256, 0, s>>>(d, x);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stream_gateup(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s) {
-  return d.qtype == MF_Q8_0 ? launch_s<kQ8, 2>(d, tm, layer, wave, T, s) : launch_s<kQ4, 2>(d, tm, layer, wave, T, s);
+cudaError_t launch_stream_gateup(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, bool overlap,
+                                 cudaStream_t s) {
+  return d.qtype == MF_Q8_0 ? launch_s<kQ8, 2>(d, tm, layer, wave, T, overlap, s)
+                            : launch_s<kQ4, 2>(d, tm, layer, wave, T, overlap, s);
 }
 
 cudaError_t launch_stream_down(const Dev& d, const CUtensorMap* tm, int layer, int wave, int T, cudaStream_t s) {
-  return d.qtype == MF_Q8_0 ? launch_s<kQ8, 1>(d, tm, layer, wave, T, s) : launch_s<kQ4, 1>(d, tm, layer, wave, T, s);
+  return d.qtype == MF_Q8_0 ? launch_s<kQ8, 1>(d, tm, layer, wave, T, true, s)
+                            : launch_s<kQ4, 1>(d, tm, layer, wave, T, true, s);
 }
 
 }  // namespace mf
