@@ -87,7 +87,7 @@ struct Carve {
 struct ScratchOffsets {
   uint64_t slot_of, expert_of, last_use, clock, stats, tr_n, tr_expert, tr_slot, tr_hit;
   uint64_t zpart, idx, g, uniq, uslot, umiss, asg_off, asg, pos_slot, info, miss_list, h, part;
-  uint64_t work, err, tb_off, sx, sb, sy, sidx, sw, stage, xs, hs, xe;
+  uint64_t work, err, tb_off, sx, sb, sy, sidx, sw, stage, xs, hs, xe, sched;
   uint64_t total;
 };
 
@@ -118,6 +118,7 @@ ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   o.h = c.take<float>(k * I);
   o.part = c.take<float>(Tm > 1 ? (uint64_t)Tm * k * H : 1);
   o.work = c.take<uint64_t>(16);  // the fused FFN's grid arrival counter, alone on its 128-byte line
+  o.sched = c.take<unsigned>(2 * (E + 1));
   o.err = c.take<unsigned>(1);
   o.tb_off = c.take<int32_t>(E + 1);
   o.sx = c.take<float>((uint64_t)Tm * H);
@@ -362,6 +363,7 @@ int create_ctx(mf_ctx_t** out, const mf_model_t* m, const mf_plan_t* p, int devi
   d.work = reinterpret_cast<unsigned long long*>(base + so.work);
   d.stage = Tm > 1 ? base + so.stage : nullptr;
   d.err = reinterpret_cast<unsigned*>(base + so.err);
+  d.sched = reinterpret_cast<unsigned*>(base + so.sched);
   d.xs = base + so.xs;
   d.hs = base + so.hs;
   d.xe = reinterpret_cast<int32_t*>(base + so.xe);

@@ -83,6 +83,7 @@ struct Dev {
   uint8_t* ht;         // h tiles:  t * (I / 32) + kk
   uint8_t* stage;      // [S_alloc] payloads: a wave's misses staged while the previous wave computes (T_max > 1)
   unsigned long long* work;  // [16]     arrival counter of the fused one-token FFN kernel (word 0)
+  unsigned* sched;     // [2 (E + 1)]   work counters of the streaming kernels: wave w's gate/up at 2w, down at 2w + 1
   unsigned* err;       // [1]           nonzero after a bounded wait gave up (see MF_E_TIMEOUT)
   uint64_t wait_ns;    // time limit of every bounded device wait (mf_wait_limit)
   int hold;            // test hold (mf_test_hold): the fused FFN's producer issues no copies

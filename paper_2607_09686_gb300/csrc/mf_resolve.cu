@@ -269,9 +269,12 @@ __global__ void __launch_bounds__(kThreadsRes, 1) k_resolve(Dev d, int layer, in
     s_expert_of[tid] = g_expert_of[tid];
     s_last[tid] = g_last[tid];
   }
-  {  // every wave the host may launch for this call starts with no misses
+  {  // every wave the host may launch for this call starts with no misses and no work drawn
     const int acc_max = n < E ? n : E;
-    if (tid < (acc_max + S - 1) / S) d.info[2 + tid] = 0;
+    if (tid < (acc_max + S - 1) / S) {
+      d.info[2 + tid] = 0;
+      d.sched[2 * tid] = d.sched[2 * tid + 1] = 0;
+    }
   }
   __syncthreads();
   // routes c0 + j * nt of this thread (j < kRouteChunk) are loaded first, then counted into

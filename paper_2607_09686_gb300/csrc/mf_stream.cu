@@ -24,8 +24,9 @@
 //
 // Work unit = (expert, 64 row records, up to 32 assignments): 128 weight rows, for gate/up 64 gate and
 // the same 64 up rows, so that one thread ends with gate and up of the same output feature.  One CTA per
-// SM takes units blockIdx.x, + gridDim.x, ... and walks each in K chunks of 128 weights: a producer warp
-// fills a ring of stages (TMA boxes of codes, 128-byte / 64-byte swizzled so that the fragment loads are
+// SM takes units one after another from a counter (their costs differ with the assignments; dealt out in
+// turn, the last SM ended 13 % after the average) and walks each in K chunks of 128 weights: a producer
+// warp fills a ring of stages (TMA boxes of codes, 128-byte / 64-byte swizzled so that the fragment loads are
 // conflict free; TMA boxes of scales; one bulk copy of 768 bytes per assignment's activation pieces), 16
 // consumer warps take 16 rows x 64 K each (8 row groups x 2 K halves of the stage) and convert the codes
 // in registers.  The halves' sums meet in shared memory once per unit.
@@ -75,11 +76,12 @@ StreamCfg stream_cfg(const Dev& d, int T) {
   c.stage = (a + (uint32_t)c.cols * kColStride + 1023) & ~1023u;
   const uint32_t red = 2u * 8 * 32 * (c.cols / 8) * 16;  // two buffers of the K halves' sums
   const uint32_t tab = (uint32_t)(3 * (d.S_active + 1)) * 4;
-  const uint32_t fixed = 1024 + 2 * kSMaxStages * 8 + red + tab;
+  const uint32_t bars = (2 * kSMaxStages + 32) * 8 + kSMaxStages * 4;
+  const uint32_t fixed = 1024 + bars + red + tab;
   const uint32_t ns = ((uint32_t)kSSmem - fixed) / c.stage;
   c.NS = ns > (uint32_t)kSMaxStages ? kSMaxStages : (int)ns;
   c.off_bar = (uint32_t)c.NS * c.stage;
-  c.off_red = c.off_bar + 2 * kSMaxStages * 8;
+  c.off_red = c.off_bar + bars;
   c.off_tab = c.off_red + red;
   c.total = c.off_tab + tab;
   return c;
@@ -94,8 +96,7 @@ __device__ __forceinline__ void tma_3d(void* dst, const CUtensorMap* tmap, int x
 }
 
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -144,78 +145,88 @@ struct SUnit {
   int z, y, a0, n;  // slot plane, first row, first assignment (into asg), assignments
 };
 
-// One unit's K loop and epilogue for one consumer warp; NTL = MMA column tiles.
+// One consumer warp's place in the ring, and its row group's exchange of the K halves' sums
+struct SRing {
+  int stage = 0, unit = 0;
+  uint32_t phase = 0;
+};
+
+// kB consecutive 32-weight blocks of one stage, from block kb: the A fragments are converted once, every
+// tile's MMAs go to fresh accumulators, the scales are applied in fp32.  All kB blocks form one straight
+// line of code: their MMA chains overlap.
+template <int QT, int NTL, int kB>
+__device__ __forceinline__ void stream_blocks(const unsigned char* st, const unsigned char* bp, const uint32_t (&off)[2],
+                                              int kb, const float (&dl)[2], const float (&dh)[2], float (&acc)[NTL][4]) {
+  uint32_t a[kB][2][4];
+#pragma unroll
+  for (int b = 0; b < kB; ++b) load_a<QT>(st + off[b], st + SL<QT>::kBox + off[b], a[b]);
+#pragma unroll
+  for (int i = 0; i < NTL; ++i) {
+#pragma unroll
+    for (int b = 0; b < kB; ++b) {
+      const unsigned char* bc = bp + (uint32_t)i * 8 * kColStride + (kb + b) * 64;
+      const uint4 v0 = *reinterpret_cast<const uint4*>(bc);
+      const uint4 v1 = *reinterpret_cast<const uint4*>(bc + kKC * 2);
+      const uint4 v2 = *reinterpret_cast<const uint4*>(bc + kKC * 4);
+      float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
+      mma16816(c, a[b][0], v0.x, v0.y);  // top pieces
+      mma16816(e, a[b][0], v2.x, v2.y);  // the others, the smallest first
+      mma16816(c, a[b][1], v0.z, v0.w);
+      mma16816(e, a[b][1], v2.z, v2.w);
+      mma16816(e, a[b][0], v1.x, v1.y);
+      mma16816(e, a[b][1], v1.z, v1.w);
+      acc[i][0] = fmaf(dl[b], c[0] + e[0], acc[i][0]);
+      acc[i][1] = fmaf(dl[b], c[1] + e[1], acc[i][1]);
+      acc[i][2] = fmaf(dh[b], c[2] + e[2], acc[i][2]);
+      acc[i][3] = fmaf(dh[b], c[3] + e[3], acc[i][3]);
+    }
+  }
+}
+
+// One unit's K loop and epilogue for one consumer warp (its first stage has arrived); NTL = MMA column
+// tiles.  False once a bounded wait gave up.
 template <int QT, int NT, int NTL>
-__device__ __forceinline__ void stream_unit(const Dev& d, const SUnit& un, unsigned char* smem, uint64_t* full,
-                                            uint64_t* empty, const StreamCfg& f, float4* red, int KC, int nb, int rows,
-                                            int& stage, uint32_t& phase, bool& ok, int warp, int lane) {
+__device__ __forceinline__ bool stream_unit(const Dev& d, const SUnit& un, unsigned char* smem, uint64_t* full,
+                                            uint64_t* empty, uint64_t* rbar, const StreamCfg& f, float4* red, int KC,
+                                            int nb, int rows, SRing& r, int warp, int lane) {
   using L = SL<QT>;
   const int grp = warp & 7, half = warp >> 3, g = lane >> 2, t = lane & 3;
   const int row = grp * 8 + g;  // record row inside each box
-  // this lane's code offset of block kb inside a box: the TMA swizzle XORs the 16-byte chunk with the row
-  auto code_off = [&](int kb) -> uint32_t {
+  uint32_t off[2];  // this lane's codes of its two blocks inside a box: the TMA swizzle XORs the 16-byte chunk with the row
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const int kb = half * 2 + b;
     if constexpr (QT == kQ8)
-      return (uint32_t)row * 128 + ((uint32_t)((kb * 2 + (t >> 1)) ^ (row & 7)) << 4) + (t & 1) * 8;
+      off[b] = (uint32_t)row * 128 + ((uint32_t)((kb * 2 + (t >> 1)) ^ (row & 7)) << 4) + (t & 1) * 8;
     else
-      return (uint32_t)row * 64 + ((uint32_t)(kb ^ ((row >> 1) & 3)) << 4) + t * 4;
-  };
-  int pos[NTL][2];  // assignments of this lane's columns, and the scale exponent of their tokens
-  int ex[NTL][2];
-#pragma unroll
-  for (int i = 0; i < NTL; ++i)
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int c = i * 8 + 2 * t + q;
-      pos[i][q] = (half == 0 && c < un.n) ? d.asg[un.a0 + c] : -1;
-      ex[i][q] = pos[i][q] < 0 ? 0 : d.xe[pos[i][q] / d.k];
-    }
+      off[b] = (uint32_t)row * 64 + ((uint32_t)(kb ^ ((row >> 1) & 3)) << 4) + t * 4;
+  }
+  int pl = -1, el = 0;  // assignment of column `lane` and the scale exponent of its token
+  if (half == 0 && lane < un.n) {
+    pl = d.asg[un.a0 + lane];
+    el = d.xe[pl / d.k];
+  }
   float acc[NTL][4], tot[NTL][4];  // sums of a segment of kSeg stages, of the row
 #pragma unroll
   for (int i = 0; i < NTL; ++i)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[i][q] = tot[i][q] = 0.f;
 
-  for (int kc = 0; ok && kc < KC; ++kc) {
-    if (!mbar_wait(&full[stage], phase, d.wait_ns)) {
-      if (lane == 0) atomicExch(d.err, 6u);
-      ok = false;
-      break;
-    }
-    const unsigned char* st = smem + (size_t)stage * f.stage;
+  for (int kc = 0; kc < KC; ++kc) {
+    if (kc > 0 && !mbar_wait(&full[r.stage], r.phase, d.wait_ns)) return false;
+    const unsigned char* st = smem + (size_t)r.stage * f.stage;
     const uint32_t so = L::kOffScale + (uint32_t)row * kScaleBoxBytes + ((kc & 1) * 2 + half) * 4;
     const __half2 s_lo = *reinterpret_cast<const __half2*>(st + so);
     const __half2 s_hi = *reinterpret_cast<const __half2*>(st + so + kRecs * kScaleBoxBytes);
     const unsigned char* bp = st + L::kOffB + (uint32_t)g * kColStride + t * 16;
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const int kb = half * 2 + b;
-      if (kc * 4 + kb < nb) {  // warp-uniform: blocks past the end of the row are skipped
-        uint32_t a[2][4];
-        const uint32_t off = code_off(kb);
-        load_a<QT>(st + off, st + L::kBox + off, a);
-        const float dl = b ? __high2float(s_lo) : __low2float(s_lo), dh = b ? __high2float(s_hi) : __low2float(s_hi);
-#pragma unroll
-        for (int i = 0; i < NTL; ++i) {
-          const unsigned char* bc = bp + (uint32_t)i * 8 * kColStride + kb * 64;
-          float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
-          const uint4 v0 = *reinterpret_cast<const uint4*>(bc);
-          const uint4 v1 = *reinterpret_cast<const uint4*>(bc + kKC * 2);
-          const uint4 v2 = *reinterpret_cast<const uint4*>(bc + kKC * 4);
-          mma16816(c, a[0], v0.x, v0.y);  // top pieces
-          mma16816(e, a[0], v2.x, v2.y);  // the others, the smallest first
-          mma16816(c, a[1], v0.z, v0.w);
-          mma16816(e, a[1], v2.z, v2.w);
-          mma16816(e, a[0], v1.x, v1.y);
-          mma16816(e, a[1], v1.z, v1.w);
-          acc[i][0] = fmaf(dl, c[0] + e[0], acc[i][0]);
-          acc[i][1] = fmaf(dl, c[1] + e[1], acc[i][1]);
-          acc[i][2] = fmaf(dh, c[2] + e[2], acc[i][2]);
-          acc[i][3] = fmaf(dh, c[3] + e[3], acc[i][3]);
-        }
-      }
-    }
+    const float dl[2] = {__low2float(s_lo), __high2float(s_lo)}, dh[2] = {__low2float(s_hi), __high2float(s_hi)};
+    const int kb = half * 2, left = nb - kc * 4 - kb;  // blocks of the row from this warp's first on
+    if (left >= 2)
+      stream_blocks<QT, NTL, 2>(st, bp, off, kb, dl, dh, acc);
+    else if (left == 1)
+      stream_blocks<QT, NTL, 1>(st, bp, off, kb, dl, dh, acc);
     __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[stage]);
+    if (lane == 0) mbar_arrive(&empty[r.stage]);
     if ((kc & (kSeg - 1)) == kSeg - 1) {
 #pragma unroll
       for (int i = 0; i < NTL; ++i)
@@ -225,9 +236,9 @@ __device__ __forceinline__ void stream_unit(const Dev& d, const SUnit& un, unsig
           acc[i][q] = 0.f;
         }
     }
-    if (++stage == f.NS) {
-      stage = 0;
-      phase ^= 1u;
+    if (++r.stage == f.NS) {
+      r.stage = 0;
+      r.phase ^= 1u;
     }
   }
 #pragma unroll
@@ -235,41 +246,51 @@ __device__ __forceinline__ void stream_unit(const Dev& d, const SUnit& un, unsig
 #pragma unroll
     for (int q = 0; q < 4; ++q) tot[i][q] += acc[i][q];
 
-  // the two K halves of a row group meet (one barrier per unit: `red` alternates between two buffers;
-  // a warp that gave up a wait still takes part)
-  float4* rp = red + (size_t)grp * 32 * NTL + lane;
-  if (half == 1)
+  // the two K halves of a row group meet: half 1 leaves its sums in one of the group's two buffers
+  const int buf = r.unit & 1;
+  const uint32_t par = (uint32_t)(r.unit >> 1) & 1u;
+  uint64_t* filled = rbar + grp * 4 + buf;
+  uint64_t* taken = filled + 2;
+  float4* rp = red + (size_t)(buf * 8 + grp) * (f.cols / 8) * 32 + lane;
+  if (half == 1) {
+    if (r.unit >= 2 && !mbar_wait(taken, par ^ 1u, d.wait_ns)) return false;
 #pragma unroll
     for (int i = 0; i < NTL; ++i) rp[i * 32] = make_float4(tot[i][0], tot[i][1], tot[i][2], tot[i][3]);
-  named_bar_sync(1 + grp, 64);
-  if (half != 0 || !ok) return;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(filled);
+    return true;
+  }
+  if (!mbar_wait(filled, par, d.wait_ns)) return false;
 #pragma unroll
   for (int i = 0; i < NTL; ++i) {
     const float4 o = rp[i * 32];
     const float v[4] = {tot[i][0] + o.x, tot[i][1] + o.y, tot[i][2] + o.z, tot[i][3] + o.w};
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      if (pos[i][q] < 0) continue;
+      const int pos = __shfl_sync(0xffffffffu, pl, i * 8 + 2 * t + q), e = __shfl_sync(0xffffffffu, el, i * 8 + 2 * t + q);
+      if (pos < 0) continue;
       if constexpr (NT == 2) {
-        const int r = un.y + row;  // v[q]: gate, v[q + 2]: up, of output feature r
-        if (r < rows) {
-          const float h = v[q] / (1.0f + expf(-dq::scale2(v[q], ex[i][q]))) * v[q + 2];
+        const int o_row = un.y + row;  // v[q]: gate, v[q + 2]: up, of output feature o_row
+        if (o_row < rows) {
+          const float h = v[q] / (1.0f + expf(-dq::scale2(v[q], e))) * v[q + 2];
           uint16_t p[3];
           split3(h, p);
-          uint16_t* hp = reinterpret_cast<uint16_t*>(d.hs + ((size_t)pos[i][q] * ((d.I + kKC - 1) / kKC) + r / kKC) * kColBytes) +
-                         ((r & (kKC - 1) & ~31) | stream_pos<QT>(r & 31));
+          uint16_t* hp = reinterpret_cast<uint16_t*>(d.hs + ((size_t)pos * ((d.I + kKC - 1) / kKC) + o_row / kKC) * kColBytes) +
+                         ((o_row & (kKC - 1) & ~31) | stream_pos<QT>(o_row & 31));
           hp[0] = p[0];
           hp[kKC] = p[1];
           hp[2 * kKC] = p[2];
         }
       } else {
-        float* o2 = d.part + (size_t)pos[i][q] * d.H + un.y + row;
-        const int e = ex[i][q];
+        float* o2 = d.part + (size_t)pos * d.H + un.y + row;
         if (un.y + row < rows) o2[0] = dq::scale2(dq::scale2(v[q], e), e);
         if (un.y + kRecs + row < rows) o2[kRecs] = dq::scale2(dq::scale2(v[q + 2], e), e);
       }
     }
   }
+  __syncwarp();
+  if (lane == 0) mbar_arrive(taken);
+  return true;
 }
 
 // NT = 2: gate and up rows of the same 64 records; NT = 1: 128 down rows (two boxes of 64 records).
@@ -281,6 +302,8 @@ __global__ void __launch_bounds__(kSThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + f.off_bar);
   uint64_t* empty = full + kSMaxStages;
+  uint64_t* rbar = empty + kSMaxStages;  // [8 row groups]: filled x 2, taken x 2
+  int* s_q = reinterpret_cast<int*>(rbar + 32);  // [kSMaxStages] the block's j-th unit at j % kSMaxStages
   float4* red = reinterpret_cast<float4*>(smem + f.off_red);
   int* s_units = reinterpret_cast<int*>(smem + f.off_tab);  // [nu + 1] units before expert i of the wave
   int* s_asg = s_units + d.S_active + 1;                    // [nu + 1] its first assignment
@@ -295,6 +318,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kSWarps);
     }
+    for (int i = 0; i < 32; ++i) mbar_init(&rbar[i], 1);
     mbar_fence_init();
   }
   pdl_wait();
@@ -332,22 +356,29 @@ __global__ void __launch_bounds__(kSThreads, 1)
     const int r = i - s_units[lo], cb = r / nrb, n = s_asg[lo + 1] - s_asg[lo] - cb * kSCols;
     return {layer * d.S_alloc + s_slot[lo], (r - cb * nrb) * kUnitRows, s_asg[lo] + cb * kSCols, min(n, kSCols)};
   };
-  const int grid = (int)gridDim.x;
 
   if (warp == kSWarps) {  // ---- producer warp
-    int stage = 0, it = 0;
+    int stage = 0, it = 0, next = (int)blockIdx.x;
     uint32_t phase = 0;
     bool ok = true;
     const uint8_t* src = NT == 2 ? d.xs : d.hs;
     const size_t cstride = (size_t)KC * kColBytes;
-    for (int i = (int)blockIdx.x; ok && i < total; i += grid) {
-      const SUnit un = unit_at(i);
+    unsigned* ctr = d.sched + 2 * wave + (NT == 1);
+    for (int j = 0; ok; ++j) {
+      const int i = next;
+      const bool end = i >= total;
+      SUnit un = {0, 0, 0, 0};
       const uint8_t* col = nullptr;  // this lane's assignment: its activation pieces
-      if (lane < un.n) {
-        const int a = __ldg(&d.asg[un.a0 + lane]);
-        col = src + (size_t)(NT == 2 ? a / d.k : a) * cstride;
+      if (!end) {
+        if (lane == 0) next = (int)gridDim.x + (int)atomicAdd(ctr, 1u);  // the unit after this one
+        un = unit_at(i);
+        if (lane < un.n) {
+          const int a = __ldg(&d.asg[un.a0 + lane]);
+          col = src + (size_t)(NT == 2 ? a / d.k : a) * cstride;
+        }
       }
-      for (int kc = 0; kc < KC; ++kc, ++it) {
+      const int n_kc = end ? 1 : KC;
+      for (int kc = 0; kc < n_kc; ++kc, ++it) {
         if (it >= f.NS) ok = mbar_wait(&empty[stage], phase ^ 1u, d.wait_ns);
         if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
@@ -355,14 +386,19 @@ __global__ void __launch_bounds__(kSThreads, 1)
         }
         unsigned char* st = smem + (size_t)stage * f.stage;
         if (lane == 0) {
-          mbar_arrive_tx(&full[stage], 2 * L::kBox + 2 * kRecs * kScaleBoxBytes + (uint32_t)un.n * kColBytes);
+          if (kc == 0) s_q[j % kSMaxStages] = end ? -1 : i;
+          if (end) {
+            mbar_arrive(&full[stage]);
+          } else {
+            mbar_arrive_tx(&full[stage], 2 * L::kBox + 2 * kRecs * kScaleBoxBytes + (uint32_t)un.n * kColBytes);
 #pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            const int x = (NT == 2 && b ? (int)d.lay.o_up : 0) + kc * (int)L::kRow;
-            const int xs = (int)(NT == 2 ? (b ? d.lay.o_us : d.lay.o_gs) : d.lay.o_ds) + (kc >> 1) * (int)kScaleBoxBytes;
-            const int y = un.y + (NT == 1 && b ? kRecs : 0);
-            tma_3d(st + b * L::kBox, &tmap, x, y, un.z, &full[stage]);
-            tma_3d(st + L::kOffScale + b * kRecs * kScaleBoxBytes, &smap, xs, y, un.z, &full[stage]);
+            for (int b = 0; b < 2; ++b) {
+              const int x = (NT == 2 && b ? (int)d.lay.o_up : 0) + kc * (int)L::kRow;
+              const int xs = (int)(NT == 2 ? (b ? d.lay.o_us : d.lay.o_gs) : d.lay.o_ds) + (kc >> 1) * (int)kScaleBoxBytes;
+              const int y = un.y + (NT == 1 && b ? kRecs : 0);
+              tma_3d(st + b * L::kBox, &tmap, x, y, un.z, &full[stage]);
+              tma_3d(st + L::kOffScale + b * kRecs * kScaleBoxBytes, &smap, xs, y, un.z, &full[stage]);
+            }
           }
         }
         __syncwarp();
@@ -372,6 +408,8 @@ __global__ void __launch_bounds__(kSThreads, 1)
           phase ^= 1u;
         }
       }
+      if (end) break;
+      next = __shfl_sync(0xffffffffu, next, 0);
     }
     if (lane == 0) {
       if (!ok) atomicExch(d.err, 1u);
@@ -379,23 +417,25 @@ __global__ void __launch_bounds__(kSThreads, 1)
       for (int s = 0; s < f.NS && s < it; ++s)
         if (!mbar_wait(&full[s], (uint32_t)((it - 1 - s) / f.NS) & 1u, d.wait_ns)) atomicExch(d.err, 2u);
     }
-  } else {  // ---- consumers
-    int stage = 0, buf = 0;
-    uint32_t phase = 0;
+  } else {  // ---- consumers: units in the order the producer drew them
+    SRing r;
     bool ok = true;
-    for (int i = (int)blockIdx.x; i < total; i += grid, buf ^= 1) {
+    while ((ok = mbar_wait(&full[r.stage], r.phase, d.wait_ns))) {
+      const int i = s_q[r.unit % kSMaxStages];
+      if (i < 0) break;
       const SUnit un = unit_at(i);
-      float4* rb = red + (size_t)buf * 8 * 32 * (f.cols / 8);
-#define MF_UNIT(N) \
-  stream_unit<QT, NT, N>(d, un, smem, full, empty, f, rb, KC, nb, rows, stage, phase, ok, warp, lane)
+#define MF_UNIT(N) stream_unit<QT, NT, N>(d, un, smem, full, empty, rbar, f, red, KC, nb, rows, r, warp, lane)
       switch ((un.n + 7) >> 3) {
-        case 1: MF_UNIT(1); break;
-        case 2: MF_UNIT(2); break;
-        case 3: MF_UNIT(3); break;
-        default: MF_UNIT(4); break;
+        case 1: ok = MF_UNIT(1); break;
+        case 2: ok = MF_UNIT(2); break;
+        case 3: ok = MF_UNIT(3); break;
+        default: ok = MF_UNIT(4); break;
       }
 #undef MF_UNIT
+      if (!ok) break;
+      ++r.unit;
     }
+    if (!ok && lane == 0) atomicExch(d.err, 6u);
   }
   __syncthreads();
 }
