@@ -280,7 +280,7 @@ struct mf_ctx {
   CUtensorMap ts_gu[2], ts_d[2];  // the same regions for the streaming kernels: [0] boxes of 64 rows' codes
                                   // of 128 weights, [1] boxes of 64 rows' 8 scales
   CUtensorMap tm_gu[2], tm_d[2];  // the slot pool's gate/up and down row records as 3-D byte tensors:
-                                  // [0] boxes of one step's codes, [1] boxes of one scale group
+                                  // [0] boxes of 128 code bytes, [1] boxes of one scale group
 };
 
 namespace mf {

@@ -5,15 +5,14 @@
 //
 // The misses are decided on the device (slot resolve), so the copy is driven by the GPU
 // itself: SMs load 16-byte vectors straight from the pinned, device-mapped pack over the
-// CPU-GPU link and store them into the slot, with no host round trip.  Launched on the
-// context's side stream, blocks stride over each missed payload of the wave in turn (with no
-// miss every block returns at once), 8 16-byte loads in flight per thread, 1.2 MB in all: the
-// link saturates at about that.  Where they go matters for the kernel computing beside them:
-// an SM with long-latency host loads outstanding serves its other blocks' memory requests
-// slowly.  So the dequantising GEMV kernels (many small blocks, scheduled as SMs free up) get
-// the copy concentrated on one SM in eight (large blocks), while the persistent GEMM kernels
-// (one block per SM with a fixed share of the work) get it spread thin over every SM.  Both
-// kernels here ask
+// CPU-GPU link and store them into the slot, with no host round trip.  Blocks stride over each
+// missed payload of the wave in turn (with no miss every block returns at once), 12 16-byte loads
+// in flight per thread.  A call of one wave has nothing beside the copy: a few large blocks on the
+// call's own stream.  In a call of several waves the copy runs on the context's side stream beside
+// the persistent expert kernels (one block per SM with a fixed share of the work): one block of 128
+// threads per SM, with at most 64 registers a thread, so that it fits beside a GEMM block (which has
+// all but 2048 registers of each SM sub-partition); 64 threads with 8 loads left the link idle
+// (4096 Q4_0 tokens on a cold 15 % cache: 2.92 ms a call, 2.59 ms this way).  The kernels here ask
 // for the largest shared-memory carveout although they use none: an SM runs blocks of one
 // carveout at a time, so only then can they share SMs with a running expert-FFN kernel (which
 // needs most of the shared memory) instead of holding those SMs until they finish.
@@ -26,18 +25,20 @@
 namespace mf {
 namespace {
 
-constexpr int kUnroll = 8;
-constexpr int kMatThreadsSpread = 64;  // one block per SM
+constexpr int kUnroll = 12;
+constexpr int kMatThreadsSpread = 128;  // one block per SM
 constexpr int kMatThreadsDense = 512;  // one block per 8 SMs
 
 // dst_stage: null to write each miss into its slot, else miss m of the wave goes to
 // dst_stage + m * stride
-__global__ void __launch_bounds__(kMatThreadsDense) k_materialize(Dev d, int layer, int wave, uint8_t* dst_stage) {
+// (Launch bounds of 1024 threads: at most 64 registers.)
+__global__ void __launch_bounds__(1024) k_materialize(Dev d, int layer, int wave, uint8_t* dst_stage) {
   pdl_trigger();
   pdl_wait();
   const int n_miss = d.info[2 + wave];
-  const size_t nvec = d.lay.stride / 16;  // 16-byte vectors per payload
-  const size_t step = (size_t)gridDim.x * blockDim.x * kUnroll;
+  const uint32_t nvec = (uint32_t)(d.lay.stride / 16);  // 16-byte vectors per payload (32-bit: registers)
+  const uint32_t step = gridDim.x * blockDim.x * kUnroll;
+#pragma unroll 1
   for (int m = 0; m < n_miss; ++m) {
     const int u = d.miss_list[wave * d.S_active + m];
     const uint4* src = reinterpret_cast<const uint4*>(
@@ -45,16 +46,17 @@ __global__ void __launch_bounds__(kMatThreadsDense) k_materialize(Dev d, int lay
                  : d.pack + ((size_t)layer * d.E + d.uniq[u]) * d.lay.stride);
     uint4* dst = reinterpret_cast<uint4*>(dst_stage ? dst_stage + (size_t)m * d.lay.stride
                                                     : d.pool + ((size_t)layer * d.S_alloc + d.uslot[u]) * d.lay.stride);
-    for (size_t i0 = (size_t)blockIdx.x * blockDim.x * kUnroll + threadIdx.x; i0 < nvec; i0 += step) {
+#pragma unroll 1
+    for (uint32_t i0 = blockIdx.x * blockDim.x * kUnroll + threadIdx.x; i0 < nvec; i0 += step) {
       uint4 v[kUnroll];
 #pragma unroll
       for (int r = 0; r < kUnroll; ++r) {  // all loads first: kUnroll transfers in flight per thread
-        const size_t i = i0 + (size_t)r * blockDim.x;
+        const uint32_t i = i0 + r * blockDim.x;
         if (i < nvec) v[r] = ld_stream(src + i);
       }
 #pragma unroll
       for (int r = 0; r < kUnroll; ++r) {
-        const size_t i = i0 + (size_t)r * blockDim.x;
+        const uint32_t i = i0 + r * blockDim.x;
         if (i < nvec) dst[i] = v[r];
       }
     }

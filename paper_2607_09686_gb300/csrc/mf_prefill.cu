@@ -17,23 +17,29 @@
 // the MMA's shared-memory order per (128-assignment block, K step of 32) -- 16 KiB tiles that
 // one bulk copy moves -- and the gate/up epilogue writes h the same way for the down GEMM.
 //
-// Work unit = (expert of the wave, block of 128 assignments, block of 128 weight rows); one
-// CTA of 14 warps per SM walks its units as a flat sequence of K steps of 32 (one quantisation
-// block), with warp-specialised roles linked by mbarriers:
-//   producer (1 warp)    per step: one TMA load per weight tensor (the 128 rows' codes of the
-//                        block, from a 3-D tensor map over the slot pool) into a 3-slot raw ring,
-//                        every 8 steps one TMA load per tensor of the rows' next 8 scales into a
-//                        2-group scale ring, and one bulk copy of the B tile into operand stage
-//                        s % 4 (lane 0 issues the copies);
-//   converters (8 warps) dequantise the raw codes exactly into the stage's A tiles (hi / lo,
-//                        no-swizzle K-major core-matrix layout): byte -> float by the
-//                        magic-number conversion, times the binary16 scale, split with packed
-//                        bf16x2 conversions;
-//   MMA (1 thread)       issues the step's tcgen05.mma (M = 128, K = 16, N = the block's assignments
-//                        rounded up to a multiple of 16) into one of two
-//                        TMEM accumulators and commits them to the stage's mbarrier;
-//   epilogue (4 warps)   reads a finished accumulator with tcgen05.ld (warp w: TMEM lanes
-//                        32 (w % 4) .. +31) while the MMAs of the next unit use the other one.
+// Work unit = (expert of the wave, block of 128 assignments, 256 weight rows as two M blocks: gate and
+// up of the same 128 records, or 256 down rows); one CTA of 27 warps per SM walks its units as a flat
+// sequence of K steps of 32 (one quantisation block), with warp-specialised roles linked by mbarriers:
+//   producer (1 warp)    per step bulk copies of the B tile into a 6-slot ring; every 128 code bytes
+//                        of K a TMA load per M block (128 rows, from a 3-D tensor map over the slot
+//                        pool) into one of 3 raw buffers; every 8 steps one TMA load per M block of
+//                        the rows' next 8 scales (lane 0 issues; a TMA box costs 2 cycles a row up to
+//                        128 bytes, so a box per step kept the copy engine as busy as the MMAs);
+//   converters (2 x 8 warps, even and odd steps) dequantise the raw codes exactly (byte -> float by the magic-number
+//                        conversion, times the binary16 scale), split with packed bf16x2
+//                        conversions and write the A operand into tensor memory (tcgen05.st; one
+//                        lane per row, hi and lo of 32 weights = 2 x 16 columns per M block);
+//   MMA (2 warps)        issue the step's tcgen05.mma, one M block each (A in tensor memory, B in shared memory;
+//                        M = 128, K = 16, N = the block's assignments rounded up to a multiple of
+//                        16) into the unit's TMEM accumulators and commits them to the slot's and
+//                        the A stage's mbarriers;
+//   epilogue (8 warps)   reads the finished accumulators with tcgen05.ld (two warps per 32 TMEM
+//                        lanes, half of the columns each); the next unit's MMAs wait for that, the
+//                        converters and copies run ahead.
+// Tensor memory: 256 columns of accumulators, 4 A stages of 64 columns.  What bounds it: the MMAs
+// (three products per weight).  With A in shared memory the MMAs' operand reads, the converters'
+// stores and the B copies together filled the shared-memory pipe (an M = 128, N = 128, K = 16 MMA
+// reads 8 KiB of it per 64 tensor cycles; down units of 128 rows also loaded a B tile per 128 rows).
 // Every wait is bounded; a wait that gives up sets the block's flag and the device error word,
 // the roles leave their loops, and the block drains its copies and MMAs (bounded) and frees
 // its tensor memory before returning.
@@ -49,18 +55,24 @@ using dq::f2_fma;
 using dq::f2_pack;
 
 constexpr int kBM = 128, kBN = 128, kBK = 32;
-constexpr int kStages = 4;  // operand stages (A + B tiles)
-constexpr int kRaw = 3;     // raw-code ring slots
+constexpr int kStages = 4;  // A operand stages in tensor memory
+constexpr int kSlots = 6;   // B ring slots
+constexpr int kRaws = 3;    // raw-code buffers, 128 code bytes of K per row each
 constexpr uint32_t kTile = kBM * kBK * 2;  // one bf16 tile: 128 rows x 32 k = 8 KiB
 constexpr uint32_t kBTile = 2 * kTile;     // B hi + lo, one bulk copy
 
-// warp roles of the 448-thread CTA
-constexpr int kConvWarps = 8;  // warps 0-7: dequantise A tiles
-constexpr int kProdWarp = 8;   // warp 8: copies
-constexpr int kMmaWarp = 9;    // warp 9, lane 0: MMA issue
-constexpr int kEpiWarp0 = 10;  // warps 10-13: epilogue; TMEM lane quarter = warp % 4
-constexpr int kThreadsW = 14 * 32;
-static_assert(kEpiWarp0 == kMmaWarp + 1 && kEpiWarp0 + 4 == kThreadsW / 32, "warp roles");
+// warp roles of the 864-thread CTA
+constexpr int kConvWarps = 8;   // warps 0-7 dequantise the even steps, 8-15 the odd ones; M block (warp / 4) % 2,
+                                // TMEM lane quarter warp % 4
+constexpr int kProdWarp = 16;   // warp 16: copies
+constexpr int kMmaWarp = 17;    // warps 17 and 18: MMA issue, one M block each
+constexpr int kEpiWarp0 = 19;   // warps 19-26: epilogue; TMEM lane quarter = warp % 4
+constexpr int kEpiWarps = 8;
+constexpr int kThreadsW = 27 * 32;
+static_assert(kEpiWarp0 == kMmaWarp + 2 && kEpiWarp0 + kEpiWarps == kThreadsW / 32, "warp roles");
+constexpr uint32_t kAcc0 = 0, kA0 = 256, kAStage = 64;  // TMEM columns: accumulators, A stages
+constexpr uint32_t kCols = 512;
+static_assert(kA0 + kStages * kAStage == kCols, "tensor memory");
 
 // Byte offset of element (row r, k) in a K-major no-swizzle tile of 128 x 32: 8x8 core
 // matrices of 128 contiguous bytes, K-adjacent core matrices 128 B apart (the descriptor's
@@ -84,21 +96,37 @@ __device__ __forceinline__ uint32_t idesc_n(int n) {
 // the MMA width of a block with n assignments: n rounded up to a multiple of 16
 __device__ __forceinline__ int n_eff(int n) { return max(16, (n + 15) & ~15); }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+// D[tmem] (+)= A[tmem] * B[smem descriptor]
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{ .reg .pred p; setp.ne.u32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+      "{ .reg .pred p; setp.ne.u32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p; }" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate));
 }
-// arrive on `bar` once every MMA this thread issued so far has completed
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+// 1 on one lane of the (converged) warp
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(r));
+  return r;
 }
+// the six MMAs of one M block and K step of 32: (hi + lo) B's hi and hi times B's lo, two K = 16 halves (of B two
+// core matrices, of A 8 columns)
+__device__ __forceinline__ void mma_step(uint32_t d_tmem, uint32_t a, uint64_t bh, uint64_t bl, uint32_t idesc,
+                                         uint32_t accumulate) {
+  constexpr uint64_t ko = 256 >> 4;
+  mma_bf16(d_tmem, a, bh, idesc, accumulate);
+  mma_bf16(d_tmem, a, bl, idesc, 1);
+  mma_bf16(d_tmem, a + 16, bh, idesc, 1);
+  mma_bf16(d_tmem, a + 8, bh + ko, idesc, 1);
+  mma_bf16(d_tmem, a + 8, bl + ko, idesc, 1);
+  mma_bf16(d_tmem, a + 24, bh + ko, idesc, 1);
+}
+// arrive on the barrier once every MMA this thread issued so far has completed
+__device__ __forceinline__ void mma_commit_at(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint64_t* bar) { mma_commit_at(smem_u32(bar)); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// generic-proxy shared-memory writes become visible to the tensor cores' (async proxy) reads
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
 // 3-D tiled TMA load of a box at (x, y, z) of `tmap` into shared memory, completing on `bar`
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tmap, int x, int y, int z, uint64_t* bar) {
   asm volatile(
@@ -143,13 +171,11 @@ __device__ __forceinline__ void split2(uint64_t w, uint32_t& hi, uint32_t& lo) {
 }
 
 // Eight byte codes c (two words; Q8_0 c = q + 128, Q4_0 nibbles masked to bytes) times the
-// scale dd = (d, d) -> one 16-byte chunk of the hi tile and of the lo tile at `off`.
+// scale dd = (d, d) -> four words of bf16 pairs of the hi part and of the lo part.
 template <uint32_t kOffBits>
-__device__ __forceinline__ void dequant8(uint32_t w0, uint32_t w1, uint64_t dd, unsigned char* hi_t,
-                                         unsigned char* lo_t, uint32_t off) {
+__device__ __forceinline__ void dequant8(uint32_t w0, uint32_t w1, uint64_t dd, uint32_t* h, uint32_t* l) {
   const uint64_t neg = f2_pack(kOffBits | 0x80000000u, kOffBits | 0x80000000u);  // -(2^23 + offset)
   const uint32_t ws[2] = {w0, w1};
-  uint32_t h[4], l[4];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const uint64_t q01 =
@@ -159,14 +185,20 @@ __device__ __forceinline__ void dequant8(uint32_t w0, uint32_t w1, uint64_t dd, 
     split2(f2_mul(q01, dd), h[2 * i], l[2 * i]);
     split2(f2_mul(q23, dd), h[2 * i + 1], l[2 * i + 1]);
   }
-  *reinterpret_cast<uint4*>(hi_t + off) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(lo_t + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
+
+// 8 consecutive columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 struct Unit {
   int u;   // unique-expert index (access order)
   int tb;  // block of 128 assignments
-  int rb;  // block of 128 weight rows
+  int rb;  // block of 128 records (gate/up) or 256 rows (down)
 };
 
 // The wave's units, expert by expert: expert u0 + e has ceil(n / 128) assignment blocks times
@@ -188,80 +220,91 @@ struct UnitMap {
   }
 };
 
-// Scales travel in groups of kGroup K steps: one 16-byte TMA box per (tensor, row) holds the
-// group's 8 binary16 scales.  A group's buffer is loaded again two groups later, once the
-// producer has seen the raw slot of a step of the group in between freed; every group but a
-// unit's last has 8 steps and the last has 4 or 8 (K is a multiple of 128), so that step lies
-// inside the group in between whenever the raw ring has at most 4 slots.
+// Scales travel in groups of kGroup K steps: one 16-byte TMA box per (M block, row) holds the
+// group's 8 binary16 scales, which the converters read into registers at their first step of the group
+// (its first or second).  A group's buffer is loaded again two groups later, once the producer has seen
+// the B slot of the step kSlots + 1 before freed: every group has 4 or 8 steps (K is a multiple of 128),
+// so that step does not lie before the second step of the buffer's previous group while kSlots <= 6.
 constexpr int kGroup = 8;
 constexpr uint32_t kScaleBox = 16;
-static_assert(kRaw <= 4 && kGroup * 2 == (int)kScaleBox, "scale groups");
+static_assert(kSlots <= 6 && kStages % 2 == 0 && kGroup * 2 == (int)kScaleBox, "scale groups");
 
-// Shared memory of one CTA: operand stages, raw ring, scale ring, barriers.
-template <int NT, int CB>  // tensors per step (2: gate and up, 1: down), code bytes per 32-weight block
-struct PLayout {
-  static constexpr int kNA = 2 * NT;                          // A tiles per stage: hi / lo per tensor
-  static constexpr uint32_t kStage = kNA * kTile + kBTile;    // + B hi / lo
-  static constexpr uint32_t kRawSlot = NT * kBM * CB;         // codes of one step (TMA boxes)
-  static constexpr uint32_t kScaleBuf = NT * kBM * kScaleBox;  // scales of one group (TMA boxes)
-  static constexpr int kBars = 2 * kRaw + 2 * kStages + 2 * 2 + 1;
-  static constexpr uint32_t kOffRaw = kStages * kStage;
-  static constexpr uint32_t kOffScale = kOffRaw + kRaw * kRawSlot;
-  static constexpr uint32_t kOffBar = kOffScale + 2 * kScaleBuf;
-  static constexpr uint32_t kOffMisc = kOffBar + kBars * 8;
-  static constexpr uint32_t kBytes = kOffMisc + 16;
-  static_assert(kRawSlot % 128 == 0 && kOffRaw % 128 == 0 && kOffScale % 128 == 0 && kScaleBuf % 128 == 0,
-                "TMA destinations are 128-byte aligned");
-};
+// Shared memory of one CTA: B ring, raw buffers (two M blocks of 128 rows x 128 code bytes, 16-byte
+// chunks XORed with the row by the TMA swizzle), scale ring, barriers.
+constexpr uint32_t kRawRow = 128;
+constexpr uint32_t kRawBuf = 2 * kBM * kRawRow;
+constexpr uint32_t kScaleBuf = 2 * kBM * kScaleBox;  // scales of one group (TMA boxes)
+constexpr int kBarFull = 0, kBarSlotFree = kSlots, kBarRawFull = 2 * kSlots, kBarRawFree = kBarRawFull + kRaws,
+              kBarSFull = kBarRawFree + kRaws, kBarAReady = kBarSFull + 2, kBarAFree = kBarAReady + 2 * kStages,
+              kBarAccFull = kBarAFree + kStages, kBarAccEmpty = kBarAccFull + 2, kBarDrain = kBarAccEmpty + 2,
+              kBars = kBarDrain + 1;
+constexpr uint32_t kOffRaw = kSlots * kBTile;
+constexpr uint32_t kOffScale = kOffRaw + kRaws * kRawBuf;
+constexpr uint32_t kOffBar = kOffScale + 2 * kScaleBuf;
+constexpr uint32_t kOffMisc = kOffBar + kBars * 8;
+constexpr uint32_t kSmemW = kOffMisc + 16;
+static_assert(kOffRaw % 1024 == 0 && kRawBuf % 1024 == 0 && kOffScale % 128 == 0 && kScaleBuf % 128 == 0,
+              "TMA destinations");
 
 // Gate/up (NT = 2) or down (NT = 1) projection of wave `wave` for every assignment of the wave.
 //   gate/up: A = gate / up rows of the slot's gate/up region, B = x tiles; epilogue
 //            h = silu(G) * U, split, into the h tiles
 //   down:    A = down rows, B = h tiles; epilogue part[assignment][hidden]
-// Pipeline (mbarriers): producer --full--> converters --a_ready--> MMA --mma_done--> producer
-// (B slot) and converters (A slot); converters --raw_free--> producer; MMA --acc_full-->
-// epilogue --acc_empty--> MMA, with two TMEM accumulators.
+// Pipeline (mbarriers): producer --raw_full--> converters --a_ready--> MMA --a_free--> converters;
+// converters --raw_free--> producer --full--> MMA --slot_free--> producer; MMA --acc_full--> epilogue
+// --acc_empty--> MMA.
+// (Launch bounds of 1024 threads: 64 registers, which leaves the materialiser room beside a GEMM block; with 72
+// its blocks waited for the GEMM's end and a cold call of several waves took 3.2 instead of 2.9 ms.)
 template <int QT, int NT>
-__global__ void __launch_bounds__(kThreadsW, 1)
+__global__ void __launch_bounds__(1024, 1)
     k_prefill(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap smap, Dev d, int layer,
               int wave) {
   constexpr int CB = QT == MF_Q8_0 ? 32 : 16;
-  using PL = PLayout<NT, CB>;
-  constexpr uint32_t kAcc = NT * kBN;  // TMEM columns of one accumulator (gate | up, or down)
-  constexpr uint32_t kCols = 2 * kAcc;
+  constexpr int RG = (int)kRawRow / CB;  // K steps of a raw buffer
   constexpr uint32_t kOffBits = QT == MF_Q8_0 ? dq::kOffQ8 : dq::kOffQ4;
   extern __shared__ __align__(1024) unsigned char smem[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + PL::kOffBar);
-  uint64_t* full = bars;                    // [kRaw]    1 expect-tx arrival (codes, scales, B tile)
-  uint64_t* raw_free = full + kRaw;         // [kRaw]    one arrival per converter warp
-  uint64_t* a_ready = raw_free + kRaw;      // [kStages] one arrival per converter warp
-  uint64_t* mma_done = a_ready + kStages;   // [kStages] tcgen05.commit
-  uint64_t* acc_full = mma_done + kStages;  // [2]       tcgen05.commit
-  uint64_t* acc_empty = acc_full + 2;       // [2]       one arrival per epilogue warp
-  uint64_t* drain = acc_empty + 2;          // [1]       tcgen05.commit
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + PL::kOffMisc);
-  volatile int* s_flag = reinterpret_cast<volatile int*>(smem + PL::kOffMisc + 4);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
+  uint64_t* full = bars + kBarFull;           // [kSlots]  1 expect-tx arrival (B tile)
+  uint64_t* slot_free = bars + kBarSlotFree;  // [kSlots]  tcgen05.commit of both MMA warps
+  uint64_t* raw_full = bars + kBarRawFull;    // [kRaws]   1 expect-tx arrival (codes)
+  uint64_t* raw_free = bars + kBarRawFree;    // [kRaws]   one arrival per converter warp
+  uint64_t* s_full = bars + kBarSFull;        // [2]       1 expect-tx arrival (a group's scales)
+  uint64_t* a_ready = bars + kBarAReady;      // [kStages][M block] one arrival per converter warp of the block
+  uint64_t* a_free = bars + kBarAFree;        // [kStages] tcgen05.commit of both MMA warps
+  uint64_t* acc_full = bars + kBarAccFull;    // [M block] tcgen05.commit
+  uint64_t* acc_empty = bars + kBarAccEmpty;  // [M block] one arrival per epilogue warp
+  uint64_t* drain = bars + kBarDrain;         // [1]       tcgen05.commit of both MMA warps
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + kOffMisc);
+  volatile int* s_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  const int K = NT == 2 ? d.H : d.I;            // reduction length
-  const int nk = K / kBK;                       // steps per unit
-  const int nrb = (NT == 2 ? d.I : d.H) / kBM;  // row blocks per expert
+  const int K = NT == 2 ? d.H : d.I;  // reduction length
+  const int nk = K / kBK;             // steps per unit
+  const int rows = NT == 2 ? d.I : d.H;
+  constexpr int kURows = NT == 2 ? kBM : 2 * kBM;  // records per unit
+  const int nrb = (rows + kURows - 1) / kURows;    // row blocks per expert
 
   // ---- prologue: barriers, tensor memory, the wave's unit prefix
   if (tid == 0) {
-    for (int i = 0; i < kRaw; ++i) {
+    for (int i = 0; i < kSlots; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&raw_free[i], kConvWarps);
+      mbar_init(&slot_free[i], 2);
     }
+    for (int i = 0; i < kRaws; ++i) {
+      mbar_init(&raw_full[i], 1);
+      mbar_init(&raw_free[i], 2 * kConvWarps);
+    }
+    for (int i = 0; i < 2; ++i) mbar_init(&s_full[i], 1);
     for (int i = 0; i < kStages; ++i) {
-      mbar_init(&a_ready[i], kConvWarps);
-      mbar_init(&mma_done[i], 1);
+      mbar_init(&a_ready[2 * i], kConvWarps / 2);
+      mbar_init(&a_ready[2 * i + 1], kConvWarps / 2);
+      mbar_init(&a_free[i], 2);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 4);
+      mbar_init(&acc_empty[i], kEpiWarps);
     }
-    mbar_init(drain, 1);
+    mbar_init(drain, 2);
     *s_flag = 0;
     mbar_fence_init();
   }
@@ -293,172 +336,198 @@ __global__ void __launch_bounds__(kThreadsW, 1)
     atomicExch(d.err, code);
     return false;
   };
-  // the same for a whole warp: lane 0 polls, the warp synchronises and shares the outcome
-  auto warp_wait = [&](uint64_t* bar, uint32_t parity, unsigned code) -> bool { return wait(bar, parity, code); };
+  // true where the unit's second M block lies past the last row (down, hidden not a multiple of 256)
+  auto half_unit = [&](const Unit& un) -> bool { return NT == 1 && un.rb * kURows + kBM >= rows; };
 
-  if (warp < kConvWarps) {
-    // ================= converters: raw codes of step s -> A tiles of stage s % kStages
-    // gate/up: thread = (tensor, row), 32 weights; down: thread = (half, row), 16 weights
-    const int r = tid & (kBM - 1), part = tid >> 7;
-    const int ten = NT == 2 ? part : 0, tr = ten * kBM + r;
-    constexpr int kGroups = NT == 2 ? 4 : 2;  // 8-weight groups of this thread
-    const int g0 = NT == 2 ? 0 : part * 2;
-    int kk = 0, slot = 0, stage = 0, gb = 1;
-    uint32_t rph = 0, sph = 0;  // phase parities of the raw ring and of the stage ring
+  if (warp < 2 * kConvWarps) {
+    // ================= converters: raw codes of step s -> A stage s % kStages; thread = (M block, row)
+    const int ten = (warp >> 2) & 1, grp = warp >> 3, tr = ten * kBM + (tid & (kBM - 1));
+    const uint32_t a_addr = tmem0 + kA0 + (uint32_t)ten * 32 + ((uint32_t)((warp & 3) * 32) << 16);
+    int kk = grp, stage = grp, gb = 1, rb = kRaws - 1;  // steps grp, grp + 2, ... (nk is even)
+    uint32_t sph = 0, gph = 1, rph = 1;  // phase parities of the A stage ring, the scale ring, the raw buffers
     uint4 sv = make_uint4(0, 0, 0, 0);  // this row's scales of the current group
-    for (int s = 0; s < n_steps; ++s) {
-      if (!warp_wait(&full[slot], rph, 1u)) break;
-      if (s >= kStages && !warp_wait(&mma_done[stage], sph ^ 1, 2u)) break;
-      const unsigned char* raw = smem + PL::kOffRaw + slot * PL::kRawSlot;
-      unsigned char* a_hi = smem + stage * PL::kStage + (2 * ten) * kTile;
-      unsigned char* a_lo = a_hi + kTile;
-      if ((kk & (kGroup - 1)) == 0) {  // first step of a group: its scales arrived with this step's codes
+    bool alive = true;
+    for (int s = grp; s < n_steps; s += 2) {
+      if ((kk & (kGroup - 1)) == grp) {  // this warp's first step of a scale group
         gb ^= 1;
-        sv = *reinterpret_cast<const uint4*>(smem + PL::kOffScale + gb * PL::kScaleBuf + tr * kScaleBox);
+        if (gb == 0) gph ^= 1;
+        if (!wait(&s_full[gb], gph, 1u)) break;
+        sv = *reinterpret_cast<const uint4*>(smem + kOffScale + gb * kScaleBuf + tr * kScaleBox);
       }
+      const int ri = kk % RG;  // the step's place in its raw buffer
+      if (ri == grp) {
+        if (++rb == kRaws) rb = 0, rph ^= 1;
+        if (!wait(&raw_full[rb], rph, 1u)) break;
+      }
+      const unsigned char* codes = smem + kOffRaw + rb * kRawBuf + (uint32_t)tr * kRawRow;
       const int q = (kk >> 1) & 3;
       const uint32_t sw = q == 0 ? sv.x : q == 1 ? sv.y : q == 2 ? sv.z : sv.w;
       const float dsc = __half2float(__ushort_as_half((unsigned short)((kk & 1) ? (sw >> 16) : (sw & 0xFFFFu))));
       const uint64_t dd = f2_pack(__float_as_uint(dsc), __float_as_uint(dsc));
-      const unsigned char* codes = raw + (size_t)tr * CB;
+      // 16 weights at a time (elements 0-15, 16-31: the two K halves of the step)
+      uint32_t w[8];
       if constexpr (QT == MF_Q8_0) {
-#pragma unroll
-        for (int g = 0; g < kGroups; ++g) {
-          const uint2 w = *reinterpret_cast<const uint2*>(codes + (g0 + g) * 8);
-          dequant8<kOffBits>(w.x, w.y, dd, a_hi, a_lo, core_off(r, (g0 + g) * 8));
-        }
+        const uint4 c0 = *reinterpret_cast<const uint4*>(codes + (((2 * ri) ^ (tr & 7)) << 4));
+        const uint4 c1 = *reinterpret_cast<const uint4*>(codes + (((2 * ri + 1) ^ (tr & 7)) << 4));
+        w[0] = c0.x, w[1] = c0.y, w[2] = c0.z, w[3] = c0.w, w[4] = c1.x, w[5] = c1.y, w[6] = c1.z, w[7] = c1.w;
       } else {
-        // byte j: element j (low nibble), element j + 16 (high nibble): groups 0 and 1 are the
-        // low nibbles of bytes 0-7 and 8-15, groups 2 and 3 their high nibbles
-        const uint4 c = *reinterpret_cast<const uint4*>(codes);
-        const uint32_t ws[4] = {c.x, c.y, c.z, c.w};
+        // byte j: element j (low nibble), element j + 16 (high nibble)
+        const uint4 c = *reinterpret_cast<const uint4*>(codes + ((ri ^ (tr & 7)) << 4));
+        w[0] = c.x, w[1] = c.y, w[2] = c.z, w[3] = c.w;
 #pragma unroll
-        for (int g = 0; g < kGroups; ++g) {
-          const int gg = g0 + g;
-          const int sh = gg >= 2 ? 4 : 0, wb = (gg & 1) * 2;
-          dequant8<kOffBits>((ws[wb] >> sh) & 0x0F0F0F0Fu, (ws[wb + 1] >> sh) & 0x0F0F0F0Fu, dd, a_hi, a_lo,
-                             core_off(r, gg * 8));
-        }
+        for (int i = 0; i < 4; ++i) w[4 + i] = (w[i] >> 4) & 0x0F0F0F0Fu, w[i] &= 0x0F0F0F0Fu;
       }
-      fence_async_smem();  // this thread's A writes, before the MMAs read them
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint32_t h[8], l[8];
+        dequant8<kOffBits>(w[4 * half], w[4 * half + 1], dd, h, l);
+        dequant8<kOffBits>(w[4 * half + 2], w[4 * half + 3], dd, h + 4, l + 4);
+        if (half == 0) {  // the MMAs have read the stage
+          if (s >= kStages && !wait(&a_free[stage], sph ^ 1, 2u)) {
+            alive = false;
+            break;
+          }
+          __syncwarp();
+          tc_fence_after();
+        }
+        tmem_st8(a_addr + stage * kAStage + half * 8, h);
+        tmem_st8(a_addr + stage * kAStage + 16 + half * 8, l);
+      }
+      if (!alive) break;
+      tmem_st_wait();
+      tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&a_ready[stage]);
-        mbar_arrive(&raw_free[slot]);
+        mbar_arrive(&a_ready[2 * stage + ten]);
+        if (ri == RG - 2 + grp || kk == nk - 2 + grp) mbar_arrive(&raw_free[rb]);  // its last step of the buffer
       }
-      if (++kk == nk) kk = 0;
-      if (++slot == kRaw) slot = 0, rph ^= 1;
-      if (++stage == kStages) stage = 0, sph ^= 1;
+      if ((kk += 2) >= nk) kk -= nk;
+      if ((stage += 2) >= kStages) stage -= kStages, sph ^= 1;
     }
   } else if (warp == kProdWarp) {
     // ================= producer (lane 0; the warp's other lanes have no role): TMA boxes of codes
     // and scales, bulk B tile
     if (lane == 0) {
-    const uint8_t* tiles = NT == 2 ? d.xt : d.ht;
-    int y0 = 0, z0 = 0;    // the unit's TMA coordinates: first row, slot plane
-    size_t b0 = 0;         // its first B tile
-    uint32_t b_bytes = 0;  // bytes of each B half the MMAs read: n_eff columns
-    int kk = 0, slot = 0, stage = 0, j = 0, gb = 1;
-    uint32_t rph = 0, sph = 0;
-    for (int s = 0; s < n_steps; ++s) {
-      if (kk == 0) {
-        const Unit un = um.at(bid + j * nb);
-        z0 = layer * d.S_alloc + d.uslot[un.u];
-        y0 = un.rb * kBM;
-        b0 = (size_t)(d.tb_off[un.u] + un.tb) * nk;
-        const int a0 = d.asg_off[un.u] + un.tb * kBN;
-        b_bytes = (uint32_t)n_eff(min(kBN, d.asg_off[un.u + 1] - a0)) * (kBK * 2);
-      }
-      if (s >= kRaw && !wait(&raw_free[slot], rph ^ 1, 3u)) break;
-      if (s >= kStages && !wait(&mma_done[stage], sph ^ 1, 4u)) break;
-      unsigned char* raw = smem + PL::kOffRaw + slot * PL::kRawSlot;
-      const bool group = (kk & (kGroup - 1)) == 0;
-      if (group) gb ^= 1;
-      {
-        mbar_arrive_tx(&full[slot], NT * kBM * CB + 2 * b_bytes + (group ? PL::kScaleBuf : 0u));
-#pragma unroll
-        for (int tn = 0; tn < NT; ++tn)
-          tma_load_3d(raw + tn * kBM * CB, &tmap, (tn ? (int)d.lay.o_up : 0) + kk * CB, y0, z0, &full[slot]);
-        if (group) {
-          // x = the scale region's start (16-byte aligned in the slot layout) + 16 bytes per group
-#pragma unroll
-          for (int tn = 0; tn < NT; ++tn) {
-            const uint32_t so = NT == 2 ? (tn ? d.lay.o_us : d.lay.o_gs) : d.lay.o_ds;
-            tma_load_3d(smem + PL::kOffScale + gb * PL::kScaleBuf + tn * kBM * kScaleBox, &smap,
-                        (int)(so + (uint32_t)(kk / kGroup) * kScaleBox), y0, z0, &full[slot]);
-          }
-        }
-        unsigned char* bdst = smem + stage * PL::kStage + PL::kNA * kTile;
-        const uint8_t* bsrc = tiles + (b0 + kk) * kBTile;
-        bulk_g2s(bdst, bsrc, b_bytes, &full[slot]);                  // hi: the first n_eff columns
-        bulk_g2s(bdst + kTile, bsrc + kTile, b_bytes, &full[slot]);  // lo
-      }
-      if (++kk == nk) kk = 0, ++j;
-      if (++slot == kRaw) slot = 0, rph ^= 1;
-      if (++stage == kStages) stage = 0, sph ^= 1;
-    }
-    }
-  } else if (warp == kMmaWarp) {
-    // ================= MMA issue (one thread)
-    if (lane == 0) {
-      int kk = 0, stage = 0, j = 0;
-      uint32_t sph = 0, idesc = 0;
+      const uint8_t* tiles = NT == 2 ? d.xt : d.ht;
+      int y0 = 0, z0 = 0;    // the unit's TMA coordinates: first row, slot plane
+      size_t b0 = 0;         // its first B tile
+      uint32_t b_bytes = 0;  // bytes of each B half the MMAs read: n_eff columns
+      int kk = 0, slot = 0, j = 0, gb = 1, rb = kRaws - 1, issued = 0, groups = 0, raws = 0;
+      uint32_t ph = 0, rph = 0;
       for (int s = 0; s < n_steps; ++s) {
-        const uint32_t acc = tmem0 + (uint32_t)(j & 1) * kAcc;
         if (kk == 0) {
           const Unit un = um.at(bid + j * nb);
+          z0 = layer * d.S_alloc + d.uslot[un.u];
+          y0 = un.rb * kURows;
+          b0 = (size_t)(d.tb_off[un.u] + un.tb) * nk;
           const int a0 = d.asg_off[un.u] + un.tb * kBN;
-          idesc = idesc_n(n_eff(min(kBN, d.asg_off[un.u + 1] - a0)));
+          b_bytes = (uint32_t)n_eff(min(kBN, d.asg_off[un.u + 1] - a0)) * (kBK * 2);
         }
-        if (kk == 0 && j >= 2 && !wait(&acc_empty[j & 1], ((j >> 1) - 1) & 1, 8u)) break;
-        if (!wait(&a_ready[stage], sph, 9u)) break;
-        tc_fence_after();
-        const uint32_t base = smem_u32(smem + stage * PL::kStage);
-        const uint64_t bh = smem_desc(base + PL::kNA * kTile), bl = smem_desc(base + PL::kNA * kTile + kTile);
-#pragma unroll
-        for (int ks = 0; ks < kBK / 16; ++ks) {
-          const uint64_t ko = (ks * 256) >> 4;  // K = 16 spans two core matrices
-#pragma unroll
-          for (int tn = 0; tn < NT; ++tn) {
-            const uint64_t ah = smem_desc(base + (2 * tn) * kTile) + ko;
-            const uint64_t al = smem_desc(base + (2 * tn + 1) * kTile) + ko;
-            const uint32_t dt = acc + tn * kBN;
-            mma_bf16(dt, ah, bh + ko, idesc, (kk | ks) != 0);
-            mma_bf16(dt, ah, bl + ko, idesc, 1);
-            mma_bf16(dt, al, bh + ko, idesc, 1);
-          }
+        const bool raw = kk % RG == 0, group = kk % kGroup == 0;
+        if (raw) {
+          if (++rb == kRaws) rb = 0, rph ^= 1;
+          if (raws >= kRaws && !wait(&raw_free[rb], rph, 3u)) break;
+          mbar_arrive_tx(&raw_full[rb], kRawBuf);
+          ++raws;
         }
-        mma_commit(&mma_done[stage]);
-        if (kk == nk - 1) mma_commit(&acc_full[j & 1]);
+        if (group) {
+          gb ^= 1;
+          mbar_arrive_tx(&s_full[gb], kScaleBuf);
+          ++groups;
+        }
+#pragma unroll
+        for (int tn = 0; tn < 2; ++tn) {  // gate and up records, or two blocks of down rows
+          const int y = y0 + (NT == 1 ? tn * kBM : 0);
+          if (raw)
+            tma_load_3d(smem + kOffRaw + rb * kRawBuf + tn * kBM * kRawRow, &tmap, (NT == 2 && tn ? (int)d.lay.o_up : 0) + kk * CB,
+                        y, z0, &raw_full[rb]);
+          // x = the scale region's start (16-byte aligned in the slot layout) + 16 bytes per group
+          const uint32_t so = NT == 2 ? (tn ? d.lay.o_us : d.lay.o_gs) : d.lay.o_ds;
+          if (group)
+            tma_load_3d(smem + kOffScale + gb * kScaleBuf + tn * kBM * kScaleBox, &smap,
+                        (int)(so + (uint32_t)(kk / kGroup) * kScaleBox), y, z0, &s_full[gb]);
+        }
+        if (s >= kSlots && !wait(&slot_free[slot], ph ^ 1, 4u)) break;
+        unsigned char* base = smem + slot * kBTile;
+        const uint8_t* bsrc = tiles + (b0 + kk) * kBTile;
+        mbar_arrive_tx(&full[slot], 2 * b_bytes);
+        bulk_g2s(base, bsrc, b_bytes, &full[slot]);                  // hi: the first n_eff columns
+        bulk_g2s(base + kTile, bsrc + kTile, b_bytes, &full[slot]);  // lo
+        ++issued;
         if (++kk == nk) kk = 0, ++j;
-        if (++stage == kStages) stage = 0, sph ^= 1;
+        if (++slot == kSlots) slot = 0, ph ^= 1;
       }
-      // nothing may be in flight when the tensor memory is freed
-      mma_commit(drain);
-      if (!mbar_wait(drain, 0, d.wait_ns)) atomicExch(d.err, 10u);
+      // no copy may be in flight when the block exits: wait for the last use of every buffer
+      for (int i = 0; i < kSlots && i < issued; ++i)
+        if (!mbar_wait(&full[i], (uint32_t)((issued - 1 - i) / kSlots) & 1u, d.wait_ns)) atomicExch(d.err, 4u);
+      for (int i = 0; i < kRaws && i < raws; ++i)
+        if (!mbar_wait(&raw_full[i], (uint32_t)((raws - 1 - i) / kRaws) & 1u, d.wait_ns)) atomicExch(d.err, 4u);
+      for (int i = 0; i < 2 && i < groups; ++i)
+        if (!mbar_wait(&s_full[i], (uint32_t)((groups - 1 - i) / 2) & 1u, d.wait_ns)) atomicExch(d.err, 4u);
     }
-  } else {
-    // ================= epilogue: accumulator j & 1 -> outputs
-    const int q4 = warp & 3;  // TMEM lanes 32 q4 .. 32 q4 + 31 = weight rows of the block
-    for (int j = 0; j < n_units; ++j) {
-      if (!warp_wait(&acc_full[j & 1], (j >> 1) & 1, 11u)) break;
+  } else if (warp < kEpiWarp0) {
+    // ================= MMA issue, one warp per M block: the whole warp walks the steps, one elected lane
+    // issues.  Warp-uniform operands stay in uniform registers: from a single thread's branch every MMA
+    // cost 72 cycles to issue whatever its N, against 64 at N = 128 and 28 at N = 16 this way.  The MMA
+    // queue is too short to cover a step's waits and commits, so two warps take turns in them.
+    const int tn = warp - kMmaWarp;
+    int kk = 0, slot = 0, stage = 0, j = 0, blocks = 2;
+    uint32_t sph = 0, ph = 0, idesc = 0;
+    const uint32_t t0 = __shfl_sync(0xffffffffu, tmem0, 0);
+    const uint32_t acc = t0 + kAcc0 + tn * kBN, smem0 = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+    const uint32_t bars0 = __shfl_sync(0xffffffffu, smem_u32(bars), 0);
+    const int steps = __shfl_sync(0xffffffffu, n_steps, 0);
+    for (int s = 0; s < steps; ++s) {
+      if (kk == 0) {
+        const Unit un = um.at(bid + j * nb);
+        const int a0 = d.asg_off[un.u] + un.tb * kBN;
+        idesc = __shfl_sync(0xffffffffu, idesc_n(n_eff(min(kBN, d.asg_off[un.u + 1] - a0))), 0);
+        blocks = __shfl_sync(0xffffffffu, half_unit(un) ? 1 : 2, 0);
+      }
+      bool ok = kk != 0 || j == 0 || wait(&acc_empty[tn], (j - 1) & 1, 8u);
+      ok = ok && wait(&full[slot], ph, 9u) && wait(&a_ready[2 * stage + tn], sph, 9u);
+      if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
+      const uint32_t base = smem0 + slot * kBTile, a0 = t0 + kA0 + stage * kAStage + tn * 32;
+      if (elect_one()) {
+        if (tn < blocks) mma_step(acc, a0, smem_desc(base), smem_desc(base + kTile), idesc, kk != 0);
+        mma_commit_at(bars0 + (uint32_t)(kBarAFree + stage) * 8);
+        mma_commit_at(bars0 + (uint32_t)(kBarSlotFree + slot) * 8);
+        if (kk == nk - 1) mma_commit_at(bars0 + (uint32_t)(kBarAccFull + tn) * 8);
+      }
+      __syncwarp();
+      if (++kk == nk) kk = 0, ++j;
+      if (++slot == kSlots) slot = 0, ph ^= 1;
+      if (++stage == kStages) stage = 0, sph ^= 1;
+    }
+    // nothing may be in flight when the tensor memory is freed
+    if (elect_one()) mma_commit(drain);
+    __syncwarp();
+    if (!mbar_wait(drain, 0, d.wait_ns)) atomicExch(d.err, 10u);
+  } else {
+    // ================= epilogue: the unit's accumulators -> outputs
+    const int q4 = warp & 3;                                     // TMEM lanes 32 q4 .. 32 q4 + 31
+    const int ch = (warp - kEpiWarp0) >> 2;                      // columns 64 ch .. 64 ch + 63
+    const uint32_t lane_addr = tmem0 + kAcc0 + ((uint32_t)(q4 * 32) << 16);
+    for (int j = 0; j < n_units; ++j) {
       const Unit un = um.at(bid + j * nb);
       const int a0 = d.asg_off[un.u] + un.tb * kBN;
-      const int n = min(kBN, d.asg_off[un.u + 1] - a0);
-      const int r = un.rb * kBM + q4 * 32 + lane;  // weight row = output feature
-      const uint32_t lane_addr = tmem0 + (uint32_t)(j & 1) * kAcc + ((uint32_t)(q4 * 32) << 16);
+      const int n = min(kBN, d.asg_off[un.u + 1] - a0), ne = n_eff(n);
       if constexpr (NT == 2) {
+        if (!wait(&acc_full[0], j & 1, 11u) || !wait(&acc_full[1], j & 1, 11u)) break;
+        __syncwarp();
+        tc_fence_after();
+        const int r = un.rb * kBM + q4 * 32 + lane;  // weight row = output feature
         // h tile of K step r / 32 of the down GEMM: this lane's row is its k = r % 32
         uint8_t* ht = d.ht + ((size_t)(d.tb_off[un.u] + un.tb) * (d.I / kBK) + (r >> 5)) * kBTile;
-        for (int c0 = 0; c0 < n_eff(n); c0 += 16) {  // the columns the down MMAs read
+        for (int c0 = ch * 64; c0 < min(ne, ch * 64 + 64); c0 += 16) {  // the columns the down MMAs read
           float g[16], u[16];
           tmem_ld16(lane_addr + c0, g);
           tmem_ld16(lane_addr + kBN + c0, u);
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             const int col = c0 + q;
-            const float hv = col < n ? g[q] / (1.0f + expf(-g[q])) * u[q] : 0.0f;
+            const float hv = col < n ? __fdividef(g[q], 1.0f + expf(-g[q])) * u[q] : 0.0f;
             const __nv_bfloat16 hi = __float2bfloat16_rn(hv);
             const uint32_t o = core_off(col, r & 31);
             *reinterpret_cast<uint16_t*>(ht + o) = __bfloat16_as_ushort(hi);
@@ -466,25 +535,43 @@ __global__ void __launch_bounds__(kThreadsW, 1)
                 __bfloat16_as_ushort(__float2bfloat16_rn(hv - __bfloat162float(hi)));
           }
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&acc_empty[0]);
+          mbar_arrive(&acc_empty[1]);
+        }
       } else {
-        for (int c0 = 0; c0 < n; c0 += 32) {
-          const int pl = c0 + lane < n ? __ldg(&d.asg[a0 + c0 + lane]) : -1;  // assignment of column c0 + lane
+        const int blocks = half_unit(un) ? 1 : 2;
+        int pl[2];  // assignments of columns 64 ch + lane and + 32
 #pragma unroll
-          for (int hlf = 0; hlf < 2; ++hlf) {
-            if (c0 + hlf * 16 >= n) break;
-            float v[16];
-            tmem_ld16(lane_addr + c0 + hlf * 16, v);
+        for (int i = 0; i < 2; ++i) pl[i] = ch * 64 + i * 32 + lane < n ? __ldg(&d.asg[a0 + ch * 64 + i * 32 + lane]) : -1;
+        bool ok = true;
+        for (int tn = 0; tn < 2; ++tn) {
+          if (!(ok = wait(&acc_full[tn], j & 1, 11u))) break;
+          __syncwarp();
+          tc_fence_after();
+          if (tn < blocks) {
+            float* out = d.part + un.rb * kURows + tn * kBM + q4 * 32 + lane;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-              const int p = __shfl_sync(0xffffffffu, pl, hlf * 16 + q);
-              if (p >= 0) d.part[(size_t)p * d.H + r] = v[q];
+            for (int hf = 0; hf < 4; ++hf) {
+              const int c0 = ch * 64 + hf * 16;
+              if (c0 >= n) break;
+              float v[16];
+              tmem_ld16(lane_addr + tn * kBN + c0, v);
+#pragma unroll
+              for (int q = 0; q < 16; ++q) {
+                const int p = __shfl_sync(0xffffffffu, pl[hf >> 1], (hf & 1) * 16 + q);
+                if (p >= 0) out[(size_t)p * d.H] = v[q];
+              }
             }
           }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[tn]);
         }
+        if (!ok) break;
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[j & 1]);
     }
   }
   tc_fence_before();
@@ -550,11 +637,10 @@ int sm_count_p() {
 
 template <int QT, int NT>
 cudaError_t launch_k(const Dev& d, const CUtensorMap* tm, int layer, int wave, cudaStream_t s) {
-  constexpr size_t smem = PLayout<NT, QT == MF_Q8_0 ? 32 : 16>::kBytes;
-  static_assert(smem <= 232448, "shared memory per block");
-  cudaError_t e = cudaFuncSetAttribute(k_prefill<QT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static_assert(kSmemW <= 232448, "shared memory per block");
+  cudaError_t e = cudaFuncSetAttribute(k_prefill<QT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemW);
   if (e != cudaSuccess) return e;
-  k_prefill<QT, NT><<<sm_count_p(), kThreadsW, smem, s>>>(tm[0], tm[1], d, layer, wave);
+  k_prefill<QT, NT><<<sm_count_p(), kThreadsW, kSmemW, s>>>(tm[0], tm[1], d, layer, wave);
   return cudaGetLastError();
 }
 
@@ -600,12 +686,12 @@ int encode_slot_region(CUtensorMap* tm, void* base, uint64_t rec_bytes, uint64_t
 
 int prefill_tensor_maps(mf_ctx* c) {
   const Dev& d = c->d;
-  const uint32_t cb = d.qtype == MF_Q8_0 ? 32 : 16;
   const uint64_t planes = (uint64_t)d.L * d.S_alloc;
-  for (int m = 0; m < 2; ++m) {  // code boxes (one step), scale boxes (one group)
-    const uint32_t box = m ? kScaleBox : cb;
-    if (encode_slot_region(&c->tm_gu[m], d.pool, d.lay.rs_gu, (uint64_t)d.I, planes, d.lay.stride, box, kBM, 0)) return -1;
-    if (encode_slot_region(&c->tm_d[m], d.pool + d.lay.d_off, d.lay.rs_d, (uint64_t)d.H, planes, d.lay.stride, box, kBM, 0))
+  for (int m = 0; m < 2; ++m) {  // code boxes (128 bytes of a row, swizzled), scale boxes (one group)
+    const uint32_t box = m ? kScaleBox : kRawRow;
+    const int sw = m ? 0 : 128;
+    if (encode_slot_region(&c->tm_gu[m], d.pool, d.lay.rs_gu, (uint64_t)d.I, planes, d.lay.stride, box, kBM, sw)) return -1;
+    if (encode_slot_region(&c->tm_d[m], d.pool + d.lay.d_off, d.lay.rs_d, (uint64_t)d.H, planes, d.lay.stride, box, kBM, sw))
       return -1;
   }
   return 0;
