@@ -104,7 +104,7 @@ ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   o.tr_expert = c.take<int32_t>(L * E);
   o.tr_slot = c.take<int32_t>(L * E);
   o.tr_hit = c.take<uint8_t>(L * E);
-  o.zpart = c.take<float2>(router_part_pairs(Tm, (int)E, (int)H));
+  o.zpart = c.take<float>(router_part_floats(Tm, (int)E, (int)H));
   o.idx = c.take<int32_t>((uint64_t)Tm * k);
   o.g = c.take<float>((uint64_t)Tm * k);
   o.uniq = c.take<int32_t>(E);
@@ -347,7 +347,7 @@ int create_ctx(mf_ctx_t** out, const mf_model_t* m, const mf_plan_t* p, int devi
   d.tr_expert = reinterpret_cast<int32_t*>(base + so.tr_expert);
   d.tr_slot = reinterpret_cast<int32_t*>(base + so.tr_slot);
   d.tr_hit = reinterpret_cast<uint8_t*>(base + so.tr_hit);
-  d.zpart = reinterpret_cast<float2*>(base + so.zpart);
+  d.zpart = reinterpret_cast<float*>(base + so.zpart);
   d.idx = reinterpret_cast<int32_t*>(base + so.idx);
   d.g = reinterpret_cast<float*>(base + so.g);
   d.uniq = reinterpret_cast<int32_t*>(base + so.uniq);

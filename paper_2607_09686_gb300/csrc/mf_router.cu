@@ -19,8 +19,8 @@
 // block 0 then runs the layer's slot resolve (lru_warp) on cache state it prefetched into
 // registers while the logits were being computed.  No global atomics or fences on the path.
 //
-// Calls with many tokens (T >= kTiledMinT) compute the logits as a tiled product instead, so
-// that W_r is read once per 32 tokens rather than once per token: see k_logits_tiled.
+// Calls with many tokens (T >= kTiledMinT) read W_r once per 64 tokens in a plain fp32 product that
+// singles out the experts that can be chosen, and compute those exactly: see k_logits_fp32.
 #include <cooperative_groups.h>
 
 #include "mf_lru.cuh"
@@ -284,41 +284,24 @@ __global__ void __launch_bounds__(kThreadsR)
 
 
 // ---------------------------------------------------------------- many tokens per call
-// k_logits_tiled: block (expert tile, token tile, K split) computes the compensated pairs of a
-// 32-token x 64-expert tile over its range of H, from shared-memory tiles of x and W_r that
-// cp.async fills 32 columns at a time (double-buffered).  Thread (ty, tx) owns tokens 2ty, 2ty+1
-// and experts tx + 16j (j < 4).  Columns are taken two at a time with f32x2 arithmetic (the same
-// IEEE operations as dot2, on two lanes): each output keeps one compensated pair for its even
-// and one for its odd columns, added error-free at the end.  The pairs of every K split go to
-// scratch; k_topk_tiled (one block per token) adds them, rounds once, adds the
-// bias, ranks and takes the softmax exactly as the one-token path does.
-constexpr int kTT = 32, kTE = 64, kHC = 32, kThreadsT = 256;
-constexpr int kPadT = kHC + 4;  // shared row stride in floats: 16 rows read together hit 2 bank phases
+// Exact (Dot2) logits are needed only for the experts that can be chosen.  k_logits_fp32 computes every
+// logit as a plain fp32 dot product (one FMA per product instead of Dot2's ten operations), k_topk_exact
+// bounds each one's error, keeps the experts whose bound reaches the k-th largest logit, and computes
+// those (k and the rare close call) with the compensated dot product, which alone decides: the routing
+// and the weights are those of exact logits for every expert.
+//
+// k_logits_fp32: block (expert tile, token tile, K split) computes a 64-token x 16 J-expert tile over its
+// range of H, from shared-memory tiles of x and W_r that cp.async fills 16 columns at a time
+// (double-buffered).  Thread (ty, tx) owns tokens 4 ty .. + 3 and experts tx + 16 j.  Columns are taken two
+// at a time with f32x2 FMAs (one running sum for the even, one for the odd columns).  The blocks of the
+// first token tile also sum the squares of the rows of W_r.
+constexpr int kTT = 64, kHC = 16, kThreadsT = 256;
+constexpr int kPadT = kHC + 4;  // shared row stride in floats: the 8 rows of a load phase use all banks
 
-__device__ __forceinline__ uint64_t f2_op_add(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_op_sub(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_op_mul(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 __device__ __forceinline__ uint64_t f2_op_fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
-}
-__device__ __forceinline__ uint64_t f2_of(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
 }
 __device__ __forceinline__ float2 f2_split(uint64_t a) {
   float lo, hi;
@@ -326,50 +309,42 @@ __device__ __forceinline__ float2 f2_split(uint64_t a) {
   return make_float2(lo, hi);
 }
 
-// dot2 on two lanes: (s, c) += a * b, product split exactly by an FMA, two-sum into s
-__device__ __forceinline__ void dot2x2(uint64_t& s, uint64_t& c, uint64_t a, uint64_t b) {
-  const uint64_t p = f2_op_mul(a, b);
-  const uint64_t pe = f2_op_fma(a, b, p ^ 0x8000000080000000ull);  // a * b - p, exact
-  const uint64_t s1 = f2_op_add(s, p);
-  const uint64_t bb = f2_op_sub(s1, s);
-  const uint64_t e = f2_op_add(f2_op_sub(s, f2_op_sub(s1, bb)), f2_op_sub(p, bb));
-  s = s1;
-  c = f2_op_add(c, f2_op_add(e, pe));
-}
-
 __device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
                : "memory");
 }
 
-__global__ void __launch_bounds__(kThreadsT)
-    k_logits_tiled(const float* __restrict__ x, const float* __restrict__ wr, int T, int E, int H, int cps,
-                   float2* __restrict__ part) {
+template <int J>
+__global__ void __launch_bounds__(kThreadsT, 2)
+    k_logits_fp32(const float* __restrict__ x, const float* __restrict__ wr, int T, int E, int H, int cps,
+                  float* __restrict__ part, float* __restrict__ wsq) {
+  constexpr int kTE = 16 * J;
   __shared__ __align__(16) float s_x[2][kTT][kPadT];
   __shared__ __align__(16) float s_w[2][kTE][kPadT];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int e0 = (int)blockIdx.x * kTE, t0 = (int)blockIdx.y * kTT;
   const int c0 = (int)blockIdx.z * cps, c1 = min(H / kHC, c0 + cps);
-  // one 16-byte piece of the x tile and two of the W tile per thread; rows past T or E read zeros
+  // one 16-byte piece of the x tile and J / 4 of the W tile per thread; rows past T or E read zeros
   auto load = [&](int ch, int buf) {
     {
-      const int r = tid >> 3, q = tid & 7, t = t0 + r;
+      const int r = tid >> 2, q = tid & 3, t = t0 + r;
       cp_async16_zfill(&s_x[buf][r][4 * q], x + (size_t)min(t, T - 1) * H + ch * kHC + 4 * q, t < T);
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int id = tid + i * kThreadsT, r = id >> 3, q = id & 7, e = e0 + r;
+    for (int i = 0; i < J / 4; ++i) {
+      const int id = tid + i * kThreadsT, r = id >> 2, q = id & 3, e = e0 + r;
       cp_async16_zfill(&s_w[buf][r][4 * q], wr + (size_t)min(e, E - 1) * H + ch * kHC + 4 * q, e < E);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   pdl_trigger();
   pdl_wait();
-  uint64_t S[2][4], C[2][4];  // [token][expert]: (even-column, odd-column) pairs
+  uint64_t S[4][J];  // [token][expert]: (even-column, odd-column) sums
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) S[a][j] = C[a][j] = 0;
+    for (int j = 0; j < J; ++j) S[a][j] = 0;
+  float sq = 0.f;  // this thread's part of its W row's square (row tid * J / 16, all columns / (16 / J))
   if (c0 < c1) load(c0, 0);
   for (int ch = c0; ch < c1; ++ch) {
     const int buf = (ch - c0) & 1;
@@ -382,115 +357,212 @@ __global__ void __launch_bounds__(kThreadsT)
     __syncthreads();
 #pragma unroll
     for (int k4 = 0; k4 < kHC; k4 += 4) {
-      const float4 xa = *reinterpret_cast<const float4*>(&s_x[buf][2 * ty][k4]);
-      const float4 xb = *reinterpret_cast<const float4*>(&s_x[buf][2 * ty + 1][k4]);
-      const uint64_t xa01 = f2_of(xa.x, xa.y), xa23 = f2_of(xa.z, xa.w);
-      const uint64_t xb01 = f2_of(xb.x, xb.y), xb23 = f2_of(xb.z, xb.w);
+      ulonglong2 xv[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 w = *reinterpret_cast<const float4*>(&s_w[buf][tx + 16 * j][k4]);
-        const uint64_t w01 = f2_of(w.x, w.y), w23 = f2_of(w.z, w.w);
-        dot2x2(S[0][j], C[0][j], w01, xa01);
-        dot2x2(S[0][j], C[0][j], w23, xa23);
-        dot2x2(S[1][j], C[1][j], w01, xb01);
-        dot2x2(S[1][j], C[1][j], w23, xb23);
+      for (int a = 0; a < 4; ++a) xv[a] = *reinterpret_cast<const ulonglong2*>(&s_x[buf][4 * ty + a][k4]);
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&s_w[buf][tx + 16 * j][k4]);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) S[a][j] = f2_op_fma(w.x, xv[a].x, S[a][j]);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) S[a][j] = f2_op_fma(w.y, xv[a].y, S[a][j]);
       }
+    }
+    if (blockIdx.y == 0) {
+      const float* w = &s_w[buf][tid * J / 16][(tid % (16 / J)) * J];
+#pragma unroll
+      for (int q = 0; q < J; ++q) sq = fmaf(w[q], w[q], sq);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    const int t = t0 + 2 * ty + a;
+  for (int a = 0; a < 4; ++a) {
+    const int t = t0 + 4 * ty + a;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < J; ++j) {
       const int e = e0 + tx + 16 * j;
-      const float2 sv = f2_split(S[a][j]), cv = f2_split(C[a][j]);
-      float ss = sv.x, cc = cv.x;
-      pair_add(ss, cc, sv.y, cv.y);
-      if (t < T && e < E) part[((size_t)blockIdx.z * T + t) * E + e] = make_float2(ss, cc);
+      const float2 v = f2_split(S[a][j]);
+      if (t < T && e < E) part[((size_t)blockIdx.z * T + t) * E + e] = v.x + v.y;
     }
+  }
+  if (blockIdx.y == 0) {
+#pragma unroll
+    for (int o = 1; o < 16 / J; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    const int e = e0 + tid * J / 16;
+    if (tid % (16 / J) == 0 && e < E) wsq[(size_t)blockIdx.z * E + e] = sq;
   }
 }
 
 constexpr int kThreadsTop = 256;
 
-// One block per token: the K splits' pairs of an expert are added by P threads (P a power of two, as
-// many as fit; each adds every P-th split in order, eight loads in flight, then thread 0 the P partial
-// pairs in order), the rest as in k_router.  (One warp per token with one load in flight at a time took
-// 87 us for the 44 splits of 64 tokens at hidden 2816 and 31 us for 4096 tokens.)
+// One block per token.  The K splits' sums of an expert are added by P threads (as many as fit, eight loads
+// in flight).  Then, with a the fp32 logit and |a - exact| <= B:
+//   a sum of H products in two chains, added over the splits, is off by less than
+//   (H / 2 + splits + 8) 2^-24 sum |x w| <= (H + 64) 2^-24 |x|_2 |w|_2 and H 2^-148 where products underflow;
+//   2^-21 of the logit's and the bias's magnitude covers the roundings after it (to fp32, the bias added).
+// L = the k-th largest of a - B is at or below the k-th largest exact logit, so an expert with a + B < L is
+// not chosen, not even on a tie.  The others are computed exactly, one warp each.  A bound that is not a
+// number (overflow) keeps its expert.
 __global__ void __launch_bounds__(kThreadsTop)
-    k_topk_tiled(Dev d, const float2* __restrict__ part, const float* __restrict__ bias, int T, int ks) {
-  __shared__ float s_z[kMaxExperts];
-  __shared__ float2 s_p[kThreadsTop];
-  __shared__ int s_sel[kMaxTopK];
-  __shared__ float s_zs[kMaxTopK];
-  const int tid = threadIdx.x, t = blockIdx.x, E = d.E, k = d.k;
+    k_topk_exact(Dev d, const float* __restrict__ x, const float* __restrict__ wr, const float* __restrict__ part,
+                 const float* __restrict__ wsq, const float* __restrict__ bias, int T, int ks) {
+  extern __shared__ __align__(16) float s_x[];  // the token's x
+  __shared__ float s_a[kMaxExperts], s_b[kMaxExperts];  // a - B, a + B; later the exact logits in s_a
+  __shared__ float s_p[2][kThreadsTop], s_n[kThreadsTop / 32];
+  __shared__ int s_cand[kMaxExperts], s_sel[kMaxTopK], s_nc, s_all;
+  __shared__ float s_zs[kMaxTopK], s_l;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, t = blockIdx.x, E = d.E, k = d.k, H = d.H;
   int P = 1;
   while (P * 2 <= ks && P * 2 * E <= kThreadsTop) P *= 2;
   const int per = kThreadsTop / P, p = tid / per;
   pdl_trigger();
   pdl_wait();
+  float nx = 0.f;
+  {
+    const float4* x4 = reinterpret_cast<const float4*>(x + (size_t)t * H);
+    for (int i = tid; i < H / 4; i += kThreadsTop) {
+      const float4 v = x4[i];
+      reinterpret_cast<float4*>(s_x)[i] = v;
+      nx += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) nx += __shfl_xor_sync(0xffffffffu, nx, o);
+  if (lane == 0) s_n[warp] = nx;
   if (tid < k) s_sel[tid] = tid;  // valid even where the logits are not ordered (NaN)
+  if (tid == 0) s_nc = s_all = 0;
+  __syncthreads();
+  nx = 0.f;
+#pragma unroll
+  for (int i = 0; i < kThreadsTop / 32; ++i) nx += s_n[i];
+  // (factors of 1.01: the roundings of the norms and of this expression)
+  const float scale = (float)(H + 64) * 0x1p-24f * 1.01f * sqrtf(nx) * 1.01f;
   for (int e0 = 0; e0 < E; e0 += per) {  // block-uniform
     const int e = e0 + tid % per;
-    float2 a = make_float2(0.f, 0.f);
+    float a = 0.f, w2 = 0.f;
     if (e < E) {
       for (int s0 = p; s0 < ks; s0 += 8 * P) {
-        float2 q[8];
+        float q[8], r[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (s0 + u * P < ks) q[u] = part[((size_t)(s0 + u * P) * T + t) * E + e];
+          if (s0 + u * P < ks) {
+            q[u] = part[((size_t)(s0 + u * P) * T + t) * E + e];
+            r[u] = wsq[(size_t)(s0 + u * P) * E + e];
+          }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (s0 + u * P < ks) pair_add(a.x, a.y, q[u].x, q[u].y);
+          if (s0 + u * P < ks) {
+            a += q[u];
+            w2 += r[u];
+          }
       }
     }
-    s_p[tid] = a;
+    s_p[0][tid] = a;
+    s_p[1][tid] = w2;
     __syncthreads();
     if (p == 0 && e < E) {
       for (int i = 1; i < P; ++i) {
-        const float2 q = s_p[tid + i * per];
-        pair_add(a.x, a.y, q.x, q.y);
+        a += s_p[0][tid + i * per];
+        w2 += s_p[1][tid + i * per];
       }
-      float v = __fadd_rn(a.x, a.y);
-      if (bias) v = __fadd_rn(v, bias[(size_t)t * E + e]);
-      s_z[e] = v;
+      const float b = bias ? bias[(size_t)t * E + e] : 0.f;
+      const float B = scale * sqrtf(w2) + 0x1p-21f * (fabsf(a) + fabsf(b)) + (float)H * 0x1p-148f;
+      s_a[e] = (a + b) - B;
+      s_b[e] = (a + b) + B;
+      if (!(fabsf(s_b[e]) < INFINITY)) s_all = 1;
     }
     __syncthreads();
   }
-  rank_topk<kThreadsTop>(s_z, E, k, s_sel, s_zs);
-  if (tid < 32) softmax_topk(d, t, k, s_sel, s_zs);
+  {  // L: the a - B of rank k - 1 (rank by counting, ties to the lower id)
+    int tpe = 1;
+    while (tpe < 32 && tpe * 2 * E <= kThreadsTop) tpe *= 2;
+    const int per_pass = kThreadsTop / tpe, q = tid % tpe;
+    for (int e0 = 0; e0 < E; e0 += per_pass) {  // block-uniform
+      const int e = e0 + tid / tpe;
+      const float z = e < E ? s_a[e] : 0.f;
+      int r = 0;
+      if (e < E)
+        for (int e2 = q; e2 < E; e2 += tpe) {
+          const float z2 = s_a[e2];
+          r += (z2 > z) || (z2 == z && e2 < e);
+        }
+      for (int off = tpe >> 1; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+      if (e < E && q == 0 && r == k - 1) s_l = z;
+    }
+  }
+  __syncthreads();
+  const float L = s_l;
+  const bool all = s_all != 0;
+  for (int e = tid; e < E; e += kThreadsTop)
+    if (all || !(s_b[e] < L)) s_cand[atomicAdd(&s_nc, 1)] = e;
+  __syncthreads();
+  const int nc = s_nc;
+  for (int c = warp; c < nc; c += kThreadsTop / 32) {
+    const float* w = wr + (size_t)s_cand[c] * H;
+    float4 pre[kChunk];
+    float zs, zc;
+    w_preload(w, H / 4, lane, 32, pre);
+    logit_part(w, s_x, H / 4, lane, 32, pre, zs, zc);
+    if (lane == 0) {
+      float z = __fadd_rn(zs, zc);
+      if (bias) z = __fadd_rn(z, bias[(size_t)t * E + s_cand[c]]);
+      s_a[c] = z;  // (the bounds in s_a are no longer read)
+    }
+  }
+  __syncthreads();
+  for (int c = tid; c < nc; c += kThreadsTop) {  // rank the candidates, ties to the lower id
+    const float z = s_a[c];
+    const int e = s_cand[c];
+    int r = 0;
+    for (int c2 = 0; c2 < nc; ++c2) r += (s_a[c2] > z) || (s_a[c2] == z && s_cand[c2] < e);
+    if (r < k) {
+      s_sel[r] = e;
+      s_zs[r] = z;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) softmax_topk(d, t, k, s_sel, s_zs);
 }
 
 // K splits for T tokens: about kTiledBlocks blocks when the tiles alone are fewer.  A constant
 // (two blocks per SM of a 152-SM part), not the device's count, so that the planner, which runs
 // without a GPU, sizes the scratch exactly as the context does.
-constexpr int kTiledBlocks = 304;
+constexpr int kTiledBlocks = 304, kMaxSplits = 64;
+int tile_experts(int E) { return E > 64 ? 128 : 64; }
 int tiled_splits(int T, int E, int H) {
-  const int tiles = ((T + kTT - 1) / kTT) * ((E + kTE - 1) / kTE);
+  const int tiles = ((T + kTT - 1) / kTT) * ((E + tile_experts(E) - 1) / tile_experts(E));
   const int nch = H / kHC;
   int want = (kTiledBlocks + tiles - 1) / tiles;
   if (want < 1) want = 1;
+  if (want > kMaxSplits) want = kMaxSplits;
   const int cps = (nch + want - 1) / want;
   return (nch + cps - 1) / cps;
 }
 
 cudaError_t launch_router_tiled(const Dev& d, const float* x, const float* wr, const float* bias, int T,
                                 cudaStream_t s) {
-  const int ks = tiled_splits(T, d.E, d.H);
+  const int ks = tiled_splits(T, d.E, d.H), te = tile_experts(d.E);
   const int nch = d.H / kHC, cps = (nch + ks - 1) / ks;
-  const cudaError_t e = launch_pdl(true, k_logits_tiled, dim3((d.E + kTE - 1) / kTE, (T + kTT - 1) / kTT, ks),
-                                   dim3(kThreadsT), 0, s, x, wr, T, d.E, d.H, cps, d.zpart);
+  float* wsq = d.zpart + (size_t)ks * T * d.E;
+  const dim3 grid((d.E + te - 1) / te, (T + kTT - 1) / kTT, ks);
+  cudaError_t e = te == 128 ? launch_pdl(true, k_logits_fp32<8>, grid, dim3(kThreadsT), 0, s, x, wr, T, d.E, d.H, cps, d.zpart, wsq)
+                            : launch_pdl(true, k_logits_fp32<4>, grid, dim3(kThreadsT), 0, s, x, wr, T, d.E, d.H, cps, d.zpart, wsq);
   if (e != cudaSuccess) return e;
-  return launch_pdl(true, k_topk_tiled, dim3(T), dim3(kThreadsTop), 0, s, d, (const float2*)d.zpart, bias, T, ks);
+  const size_t smem = (size_t)d.H * sizeof(float);
+  if (smem > 24 * 1024 &&
+      (e = cudaFuncSetAttribute(k_topk_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return e;
+  return launch_pdl(true, k_topk_exact, dim3(T), dim3(kThreadsTop), smem, s, d, x, wr, (const float*)d.zpart,
+                    (const float*)wsq, bias, T, ks);
 }
 
 }  // namespace
 
-size_t router_part_pairs(int T_max, int E, int H) {
+size_t router_part_floats(int T_max, int E, int H) {
   size_t most = 0;
   for (int T = kTiledMinT; T <= T_max; ++T) {
-    const size_t n = (size_t)tiled_splits(T, E, H) * T * E;
+    const size_t n = (size_t)tiled_splits(T, E, H) * ((size_t)T + 1) * E;
     if (n > most) most = n;
   }
   return most;

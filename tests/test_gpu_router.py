@@ -89,3 +89,24 @@ def test_router_paths_agree_at_the_switch():
         assert np.array_equal(w15, w16[:15])
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("E,T", [(40, 16), (128, 65), (200, 33)])
+def test_tiled_router_orders_logits_that_fp32_sums_cannot(E, T):
+    """Router rows that differ from one another by a few units in the last place of a few weights: the
+    logits agree to more digits than a plain fp32 sum of 1024 products keeps, so only the compensated
+    dot product orders them as the oracle does."""
+    H, k = 1024, 5
+    shape = Shape(1, H, E, k, 64, synth.Q8_0, model_seed=9)
+    ctx = Ctx(shape, slots=E, max_tokens=T)
+    try:
+        rng = np.random.default_rng(E)
+        w = np.tile(ctx.wr_host[0][:1], (E, 1))
+        for e in range(1, E):  # 3 of the weights one to four units in the last place away
+            at = rng.integers(0, H, 3)
+            w[e, at] = (w[e, at].view(np.int32) + rng.integers(-4, 5, 3).astype(np.int32)).view(np.float32)
+        ctx.wr_host[0] = w
+        ctx.wr[0] = ctx.torch.from_numpy(w).to(ctx.device)
+        _check_routes(ctx, synth.activations(23, 0, 0, 0, T, H), None, T, k)
+    finally:
+        ctx.close()
