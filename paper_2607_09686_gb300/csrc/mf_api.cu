@@ -212,6 +212,18 @@ void free_ctx(mf_ctx* c) {
   delete c;
 }
 
+// The device address of a pinned, 4-byte aligned host buffer; null for any other (pageable memory that the
+// GPU can address too: a copy to it keeps the call from returning early).
+void* pinned_target(void* p) {
+  cudaPointerAttributes a;
+  if (!p || ((uintptr_t)p & 3)) return nullptr;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+}
+
 // Repack one canonical GGUF tensor [rows x cols] into row records: the codes of row r go to
 // rec0 + r * rstride + codes_off, its binary16 scales to rec0 + r * rstride + scales_off.
 // Q8_0 codes are stored offset to unsigned (q + 128), which the dequantising kernels expect.
@@ -538,7 +550,11 @@ int mf_moe_forward(mf_ctx_t* c, int layer, const float* x, const float* router_w
   DevGuard guard(c->device);
   if (!guard.ok) return cuda_fail(cudaSetDevice(c->device), "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const Dev& d = c->d;
+  Dev d = c->d;
+  // the router stores the caller's indices and weights itself; buffers that are not aligned to their
+  // 4-byte values are copied to after the call's kernels
+  if (!((uintptr_t)idx_out & 3)) d.idx_out = idx_out, idx_out = nullptr;
+  if (!((uintptr_t)w_out & 3)) d.w_out = w_out, w_out = nullptr;
   const int S = d.S_active;
 
   timer_mark(c, kTRouter, 0, s);
@@ -685,8 +701,12 @@ int mf_moe_forward_host(mf_ctx_t* c, int layer, const float* x, const float* rou
     if (!pinned) cudaGetLastError();  // pageable memory: not an error, the copy path below serves it
     if (pinned && !(reinterpret_cast<uintptr_t>(xd) & 15)) {
       if (__atomic_load_n(&c->n_put, __ATOMIC_ACQUIRE) != (int64_t)d.L * d.E) return MF_E_STATE;
+      Dev dd = d;
+      // pinned outputs are stored by the router; others are copied to, which returns once they have arrived
+      if (void* p = pinned_target(idx_out)) dd.idx_out = static_cast<int32_t*>(p), idx_out = nullptr;
+      if (void* p = pinned_target(w_out)) dd.w_out = static_cast<float*>(p), w_out = nullptr;
       timer_mark(c, kTRouter, 0, s);
-      MF_CUDA(launch_router(d, static_cast<const float*>(xd), router_w, static_cast<const float*>(bd), 1, layer, s,
+      MF_CUDA(launch_router(dd, static_cast<const float*>(xd), router_w, static_cast<const float*>(bd), 1, layer, s,
                             c->stage_x));
       timer_mark(c, kTRouter, 1, s);
       timer_mark(c, kTFfn, 0, s);

@@ -62,6 +62,8 @@ struct Dev {
                        // [K split][E]
   int32_t* idx;        // [T_max][k]
   float* g;            // [T_max][k]
+  int32_t* idx_out;    // the caller's copies of idx and g (null: none), written by the kernel that chooses
+  float* w_out;
   int32_t* uniq;       // [E]           distinct experts in access order
   int32_t* uslot;      // [E]           their slots
   int32_t* umiss;      // [E]           1 if the access missed

@@ -152,8 +152,11 @@ __device__ __forceinline__ void softmax_topk(const Dev& d, int t, int k, const i
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
   if (lane < k) {
-    d.idx[(size_t)t * k + lane] = s_sel[lane];
-    d.g[(size_t)t * k + lane] = ex / den;
+    const size_t at = (size_t)t * k + lane;
+    d.idx[at] = s_sel[lane];
+    d.g[at] = ex / den;
+    if (d.idx_out) d.idx_out[at] = s_sel[lane];
+    if (d.w_out) d.w_out[at] = ex / den;
   }
 }
 
@@ -404,7 +407,7 @@ constexpr int kThreadsTop = 256;
 // L = the k-th largest of a - B is at or below the k-th largest exact logit, so an expert with a + B < L is
 // not chosen, not even on a tie.  The others are computed exactly, one warp each.  A bound that is not a
 // number (overflow) keeps its expert.
-__global__ void __launch_bounds__(kThreadsTop)
+__global__ void __launch_bounds__(kThreadsTop, 4)
     k_topk_exact(Dev d, const float* __restrict__ x, const float* __restrict__ wr, const float* __restrict__ part,
                  const float* __restrict__ wsq, const float* __restrict__ bias, int T, int ks) {
   extern __shared__ __align__(16) float s_x[];  // the token's x
@@ -500,10 +503,26 @@ __global__ void __launch_bounds__(kThreadsTop)
   const int nc = s_nc;
   for (int c = warp; c < nc; c += kThreadsTop / 32) {
     const float* w = wr + (size_t)s_cand[c] * H;
-    float4 pre[kChunk];
-    float zs, zc;
-    w_preload(w, H / 4, lane, 32, pre);
-    logit_part(w, s_x, H / 4, lane, 32, pre, zs, zc);
+    const float4* w4 = reinterpret_cast<const float4*>(w);
+    const float4* x4 = reinterpret_cast<const float4*>(s_x);
+    float zs = 0.f, zc = 0.f;
+    for (int q0 = lane; q0 < H / 4; q0 += 4 * 32) {  // four loads in flight: few registers, many blocks
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (q0 + u * 32 < H / 4) v[u] = ld_hint(w4 + q0 + u * 32, l2_evict_last());
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (q0 + u * 32 < H / 4) {
+          const float4 xv = x4[q0 + u * 32];
+          dot2(zs, zc, v[u].x, xv.x);
+          dot2(zs, zc, v[u].y, xv.y);
+          dot2(zs, zc, v[u].z, xv.z);
+          dot2(zs, zc, v[u].w, xv.w);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) pair_add(zs, zc, __shfl_xor_sync(0xffffffffu, zs, o), __shfl_xor_sync(0xffffffffu, zc, o));
     if (lane == 0) {
       float z = __fadd_rn(zs, zc);
       if (bias) z = __fadd_rn(z, bias[(size_t)t * E + s_cand[c]]);
