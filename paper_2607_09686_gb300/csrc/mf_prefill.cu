@@ -25,10 +25,10 @@
 //                        pool) into one of 3 raw buffers; every 8 steps one TMA load per M block of
 //                        the rows' next 8 scales (lane 0 issues; a TMA box costs 2 cycles a row up to
 //                        128 bytes, so a box per step kept the copy engine as busy as the MMAs);
-//   converters (2 x 8 warps, even and odd steps) dequantise the raw codes exactly (byte -> float by the magic-number
-//                        conversion, times the binary16 scale), split with packed bf16x2
-//                        conversions and write the A operand into tensor memory (tcgen05.st; one
-//                        lane per row, hi and lo of 32 weights = 2 x 16 columns per M block);
+//   converters (2 x 8 warps, even and odd steps) turn the raw codes into exact bf16 integers, form
+//                        hi and lo of their products with the scale in packed bf16 arithmetic and
+//                        write the A operand into tensor memory (tcgen05.st; one lane per row, hi and
+//                        lo of 32 weights = 2 x 16 columns per M block);
 //   MMA (2 warps)        issue the step's tcgen05.mma, one M block each (A in tensor memory, B in shared memory;
 //                        M = 128, K = 16, N = the block's assignments rounded up to a multiple of
 //                        16) into the unit's TMEM accumulators and commits them to the slot's and
@@ -50,7 +50,6 @@
 namespace mf {
 namespace {
 
-using dq::f2_add;
 using dq::f2_fma;
 using dq::f2_pack;
 
@@ -151,12 +150,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 
 __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 // Two values (packed fp32 pair) -> bf16x2 words hi = bf16(v), lo = bf16(v - hi).
 __device__ __forceinline__ void split2(uint64_t w, uint32_t& hi, uint32_t& lo) {
   uint32_t a, b;
@@ -170,21 +163,32 @@ __device__ __forceinline__ void split2(uint64_t w, uint32_t& hi, uint32_t& lo) {
   lo = bf2_bits(__floats2bfloat162_rn(__uint_as_float(ra), __uint_as_float(rb)));
 }
 
-// Eight byte codes c (two words; Q8_0 c = q + 128, Q4_0 nibbles masked to bytes) times the
-// scale dd = (d, d) -> four words of bf16 pairs of the hi part and of the lo part.
-template <uint32_t kOffBits>
-__device__ __forceinline__ void dequant8(uint32_t w0, uint32_t w1, uint64_t dd, uint32_t* h, uint32_t* l) {
-  const uint64_t neg = f2_pack(kOffBits | 0x80000000u, kOffBits | 0x80000000u);  // -(2^23 + offset)
-  const uint32_t ws[2] = {w0, w1};
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const uint64_t q01 =
-        f2_add(f2_pack(__byte_perm(ws[i], 0x4B000000u, 0x7650), __byte_perm(ws[i], 0x4B000000u, 0x7651)), neg);
-    const uint64_t q23 =
-        f2_add(f2_pack(__byte_perm(ws[i], 0x4B000000u, 0x7652), __byte_perm(ws[i], 0x4B000000u, 0x7653)), neg);
-    split2(f2_mul(q01, dd), h[2 * i], l[2 * i]);
-    split2(f2_mul(q23, dd), h[2 * i + 1], l[2 * i + 1]);
-  }
+// A pair of codes q (exact bf16) times the scale d = dh + dl (both bf16, exact: 11 bits) -> the bf16 parts
+// hi = RN(q d), lo = RN(q d - hi) of the weights, in four packed instructions of the FMA pipe: q dh - hi is
+// exact (it fits 8 bits), so each part is rounded once (hi to within 2^-9 of its last place of that for
+// Q8_0, whose q dl is rounded first; hi + lo is as close to q d as before, 1.2e-6 of it in the mean square).
+// Converting q d to fp32 and splitting it there kept the ALU pipe busy with byte permutes and unpacking.
+__device__ __forceinline__ void split_pair(uint32_t q, uint32_t dh, uint32_t dl, uint32_t& hi, uint32_t& lo) {
+  asm("{ .reg .b32 t, n, e;\n"
+      "mul.rn.bf16x2 t, %2, %4;\n"
+      "fma.rn.bf16x2 %0, %2, %3, t;\n"
+      "neg.bf16x2 n, %0;\n"
+      "fma.rn.bf16x2 e, %2, %3, n;\n"
+      "fma.rn.bf16x2 %1, %2, %4, e; }"
+      : "=&r"(hi), "=r"(lo)
+      : "r"(q), "r"(dh), "r"(dl));
+}
+
+// Four codes (Q8_0: bytes q + 128; Q4_0: nibbles masked to bytes) -> two words of hi and of lo.
+template <int QT>
+__device__ __forceinline__ void dequant4(uint32_t w, uint32_t dh, uint32_t dl, uint32_t* h, uint32_t* l) {
+  uint32_t q01, q23;
+  if constexpr (QT == MF_Q8_0)
+    dq::codes_q8(w, q01, q23);
+  else
+    dq::codes_q4(w, q01, q23);
+  split_pair(q01, dh, dl, h[0], l[0]);
+  split_pair(q23, dh, dl, h[1], l[1]);
 }
 
 // 8 consecutive columns of this thread's TMEM lane
@@ -234,9 +238,8 @@ static_assert(kSlots <= 6 && kStages % 2 == 0 && kGroup * 2 == (int)kScaleBox, "
 constexpr uint32_t kRawRow = 128;
 constexpr uint32_t kRawBuf = 2 * kBM * kRawRow;
 constexpr uint32_t kScaleBuf = 2 * kBM * kScaleBox;  // scales of one group (TMA boxes)
-constexpr int kBarFull = 0, kBarSlotFree = kSlots, kBarRawFull = 2 * kSlots, kBarRawFree = kBarRawFull + kRaws,
-              kBarSFull = kBarRawFree + kRaws, kBarAReady = kBarSFull + 2, kBarAFree = kBarAReady + 2 * kStages,
-              kBarAccFull = kBarAFree + kStages, kBarAccEmpty = kBarAccFull + 2, kBarDrain = kBarAccEmpty + 2,
+constexpr int kBarFull = 0, kBarDone = kSlots, kBarRawFull = 2 * kSlots, kBarRawFree = kBarRawFull + kRaws,
+              kBarSFull = kBarRawFree + kRaws, kBarAReady = kBarSFull + 2, kBarAccFull = kBarAReady + 2 * kStages, kBarAccEmpty = kBarAccFull + 2, kBarDrain = kBarAccEmpty + 2,
               kBars = kBarDrain + 1;
 constexpr uint32_t kOffRaw = kSlots * kBTile;
 constexpr uint32_t kOffScale = kOffRaw + kRaws * kRawBuf;
@@ -250,9 +253,8 @@ static_assert(kOffRaw % 1024 == 0 && kRawBuf % 1024 == 0 && kOffScale % 128 == 0
 //   gate/up: A = gate / up rows of the slot's gate/up region, B = x tiles; epilogue
 //            h = silu(G) * U, split, into the h tiles
 //   down:    A = down rows, B = h tiles; epilogue part[assignment][hidden]
-// Pipeline (mbarriers): producer --raw_full--> converters --a_ready--> MMA --a_free--> converters;
-// converters --raw_free--> producer --full--> MMA --slot_free--> producer; MMA --acc_full--> epilogue
-// --acc_empty--> MMA.
+// Pipeline (mbarriers): producer --raw_full--> converters --a_ready--> MMA --done--> converters, producer;
+// converters --raw_free--> producer --full--> MMA; MMA --acc_full--> epilogue --acc_empty--> MMA.
 // (Launch bounds of 1024 threads: 64 registers, which leaves the materialiser room beside a GEMM block; with 72
 // its blocks waited for the GEMM's end and a cold call of several waves took 3.2 instead of 2.9 ms.)
 template <int QT, int NT>
@@ -261,16 +263,14 @@ __global__ void __launch_bounds__(1024, 1)
               int wave) {
   constexpr int CB = QT == MF_Q8_0 ? 32 : 16;
   constexpr int RG = (int)kRawRow / CB;  // K steps of a raw buffer
-  constexpr uint32_t kOffBits = QT == MF_Q8_0 ? dq::kOffQ8 : dq::kOffQ4;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
   uint64_t* full = bars + kBarFull;           // [kSlots]  1 expect-tx arrival (B tile)
-  uint64_t* slot_free = bars + kBarSlotFree;  // [kSlots]  tcgen05.commit of both MMA warps
+  uint64_t* done = bars + kBarDone;           // [kSlots]  tcgen05.commit of both MMA warps: the step's slot and A stage are free
   uint64_t* raw_full = bars + kBarRawFull;    // [kRaws]   1 expect-tx arrival (codes)
   uint64_t* raw_free = bars + kBarRawFree;    // [kRaws]   one arrival per converter warp
   uint64_t* s_full = bars + kBarSFull;        // [2]       1 expect-tx arrival (a group's scales)
   uint64_t* a_ready = bars + kBarAReady;      // [kStages][M block] one arrival per converter warp of the block
-  uint64_t* a_free = bars + kBarAFree;        // [kStages] tcgen05.commit of both MMA warps
   uint64_t* acc_full = bars + kBarAccFull;    // [M block] tcgen05.commit
   uint64_t* acc_empty = bars + kBarAccEmpty;  // [M block] one arrival per epilogue warp
   uint64_t* drain = bars + kBarDrain;         // [1]       tcgen05.commit of both MMA warps
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(1024, 1)
   if (tid == 0) {
     for (int i = 0; i < kSlots; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&slot_free[i], 2);
+      mbar_init(&done[i], 2);
     }
     for (int i = 0; i < kRaws; ++i) {
       mbar_init(&raw_full[i], 1);
@@ -298,7 +298,6 @@ __global__ void __launch_bounds__(1024, 1)
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&a_ready[2 * i], kConvWarps / 2);
       mbar_init(&a_ready[2 * i + 1], kConvWarps / 2);
-      mbar_init(&a_free[i], 2);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&acc_full[i], 1);
@@ -344,7 +343,8 @@ __global__ void __launch_bounds__(1024, 1)
     const int ten = (warp >> 2) & 1, grp = warp >> 3, tr = ten * kBM + (tid & (kBM - 1));
     const uint32_t a_addr = tmem0 + kA0 + (uint32_t)ten * 32 + ((uint32_t)((warp & 3) * 32) << 16);
     int kk = grp, stage = grp, gb = 1, rb = kRaws - 1;  // steps grp, grp + 2, ... (nk is even)
-    uint32_t sph = 0, gph = 1, rph = 1;  // phase parities of the A stage ring, the scale ring, the raw buffers
+    int before = grp;                    // slot of the step kStages before (from step kStages on)
+    uint32_t bph = 0, gph = 1, rph = 1;  // phase parities of that slot, the scale ring, the raw buffers
     uint4 sv = make_uint4(0, 0, 0, 0);  // this row's scales of the current group
     bool alive = true;
     for (int s = grp; s < n_steps; s += 2) {
@@ -363,7 +363,8 @@ __global__ void __launch_bounds__(1024, 1)
       const int q = (kk >> 1) & 3;
       const uint32_t sw = q == 0 ? sv.x : q == 1 ? sv.y : q == 2 ? sv.z : sv.w;
       const float dsc = __half2float(__ushort_as_half((unsigned short)((kk & 1) ? (sw >> 16) : (sw & 0xFFFFu))));
-      const uint64_t dd = f2_pack(__float_as_uint(dsc), __float_as_uint(dsc));
+      const __nv_bfloat16 dhb = __float2bfloat16_rn(dsc), dlb = __float2bfloat16_rn(dsc - __bfloat162float(dhb));
+      const uint32_t dh = __bfloat16_as_ushort(dhb) * 0x10001u, dl = __bfloat16_as_ushort(dlb) * 0x10001u;
       // 16 weights at a time (elements 0-15, 16-31: the two K halves of the step)
       uint32_t w[8];
       if constexpr (QT == MF_Q8_0) {
@@ -380,12 +381,15 @@ __global__ void __launch_bounds__(1024, 1)
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         uint32_t h[8], l[8];
-        dequant8<kOffBits>(w[4 * half], w[4 * half + 1], dd, h, l);
-        dequant8<kOffBits>(w[4 * half + 2], w[4 * half + 3], dd, h + 4, l + 4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dequant4<QT>(w[4 * half + i], dh, dl, h + 2 * i, l + 2 * i);
         if (half == 0) {  // the MMAs have read the stage
-          if (s >= kStages && !wait(&a_free[stage], sph ^ 1, 2u)) {
-            alive = false;
-            break;
+          if (s >= kStages) {
+            if (!wait(&done[before], bph, 2u)) {
+              alive = false;
+              break;
+            }
+            if ((before += 2) >= kSlots) before -= kSlots, bph ^= 1;
           }
           __syncwarp();
           tc_fence_after();
@@ -402,7 +406,7 @@ __global__ void __launch_bounds__(1024, 1)
         if (ri == RG - 2 + grp || kk == nk - 2 + grp) mbar_arrive(&raw_free[rb]);  // its last step of the buffer
       }
       if ((kk += 2) >= nk) kk -= nk;
-      if ((stage += 2) >= kStages) stage -= kStages, sph ^= 1;
+      if ((stage += 2) >= kStages) stage -= kStages;
     }
   } else if (warp == kProdWarp) {
     // ================= producer (lane 0; the warp's other lanes have no role): TMA boxes of codes
@@ -447,7 +451,7 @@ __global__ void __launch_bounds__(1024, 1)
             tma_load_3d(smem + kOffScale + gb * kScaleBuf + tn * kBM * kScaleBox, &smap,
                         (int)(so + (uint32_t)(kk / kGroup) * kScaleBox), y, z0, &s_full[gb]);
         }
-        if (s >= kSlots && !wait(&slot_free[slot], ph ^ 1, 4u)) break;
+        if (s >= kSlots && !wait(&done[slot], ph ^ 1, 4u)) break;
         unsigned char* base = smem + slot * kBTile;
         const uint8_t* bsrc = tiles + (b0 + kk) * kBTile;
         mbar_arrive_tx(&full[slot], 2 * b_bytes);
@@ -471,31 +475,35 @@ __global__ void __launch_bounds__(1024, 1)
     // cost 72 cycles to issue whatever its N, against 64 at N = 128 and 28 at N = 16 this way.  The MMA
     // queue is too short to cover a step's waits and commits, so two warps take turns in them.
     const int tn = warp - kMmaWarp;
-    int kk = 0, slot = 0, stage = 0, j = 0, blocks = 2;
-    uint32_t sph = 0, ph = 0, idesc = 0;
+    int kk = 0, slot = 0, stage = 0, j = 0;
+    uint32_t sph = 0, ph = 0, idesc = 0, next = 0;  // instruction descriptor of the unit (0: this M block is empty), of the next
     const uint32_t t0 = __shfl_sync(0xffffffffu, tmem0, 0);
     const uint32_t acc = t0 + kAcc0 + tn * kBN, smem0 = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
     const uint32_t bars0 = __shfl_sync(0xffffffffu, smem_u32(bars), 0);
     const int steps = __shfl_sync(0xffffffffu, n_steps, 0);
+    auto unit_desc = [&](int i) -> uint32_t {
+      const Unit un = um.at(bid + i * nb);
+      const int a0 = d.asg_off[un.u] + un.tb * kBN;
+      const uint32_t v = idesc_n(n_eff(min(kBN, d.asg_off[un.u + 1] - a0)));
+      return __shfl_sync(0xffffffffu, tn == 1 && half_unit(un) ? 0u : v, 0);
+    };
+    if (steps > 0) next = unit_desc(0);
     for (int s = 0; s < steps; ++s) {
-      if (kk == 0) {
-        const Unit un = um.at(bid + j * nb);
-        const int a0 = d.asg_off[un.u] + un.tb * kBN;
-        idesc = __shfl_sync(0xffffffffu, idesc_n(n_eff(min(kBN, d.asg_off[un.u + 1] - a0))), 0);
-        blocks = __shfl_sync(0xffffffffu, half_unit(un) ? 1 : 2, 0);
-      }
+      if (kk == 0) idesc = next;
       bool ok = kk != 0 || j == 0 || wait(&acc_empty[tn], (j - 1) & 1, 8u);
-      ok = ok && wait(&full[slot], ph, 9u) && wait(&a_ready[2 * stage + tn], sph, 9u);
+      // both barriers polled at once: their latencies overlap
+      const bool f = mbar_try_wait(&full[slot], ph), a = mbar_try_wait(&a_ready[2 * stage + tn], sph);
+      ok = ok && (f || wait(&full[slot], ph, 9u)) && (a || wait(&a_ready[2 * stage + tn], sph, 9u));
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       const uint32_t base = smem0 + slot * kBTile, a0 = t0 + kA0 + stage * kAStage + tn * 32;
       if (elect_one()) {
-        if (tn < blocks) mma_step(acc, a0, smem_desc(base), smem_desc(base + kTile), idesc, kk != 0);
-        mma_commit_at(bars0 + (uint32_t)(kBarAFree + stage) * 8);
-        mma_commit_at(bars0 + (uint32_t)(kBarSlotFree + slot) * 8);
+        if (idesc) mma_step(acc, a0, smem_desc(base), smem_desc(base + kTile), idesc, kk != 0);
+        mma_commit_at(bars0 + (uint32_t)(kBarDone + slot) * 8);
         if (kk == nk - 1) mma_commit_at(bars0 + (uint32_t)(kBarAccFull + tn) * 8);
       }
       __syncwarp();
+      if (kk == 0 && j + 1 < n_units) next = unit_desc(j + 1);  // while this unit's MMAs run
       if (++kk == nk) kk = 0, ++j;
       if (++slot == kSlots) slot = 0, ph ^= 1;
       if (++stage == kStages) stage = 0, sph ^= 1;
@@ -605,9 +613,13 @@ __global__ void __launch_bounds__(256) k_tile_x(Dev d, const float* __restrict__
   __syncthreads();
   const int nk = d.H / kBK;
   uint8_t* tile0 = d.xt + (size_t)t * nk * kBTile;
-  // item i = (column i >> 2, 8-value group i & 3) of one K step: 512 per step
-  for (int it = threadIdx.x; it < nk * 512; it += blockDim.x) {
-    const int kk = it >> 9, i = it & 511, col = i >> 2, g = i & 3;
+  // item i = (column i >> 2, 8-value group i & 3) of one K step
+  const int per = n_eff(n) * 4;  // items of a K step: the columns the MMAs read
+  int kk = threadIdx.x / per, i = threadIdx.x % per;
+  for (; kk < nk; i += blockDim.x) {
+    while (i >= per) i -= per, ++kk;
+    if (kk >= nk) break;
+    const int col = i >> 2, g = i & 3;
     uint32_t h[4] = {0, 0, 0, 0}, l[4] = {0, 0, 0, 0};
     const int row = s_row[col];
     if (row >= 0) {

@@ -40,6 +40,8 @@
 namespace mf {
 namespace {
 
+using dq::codes_q4;
+using dq::codes_q8;
 using dq::kQ4;
 using dq::kQ8;
 
@@ -99,25 +101,6 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ uint32_t bf2_sub(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
-}
-
-// Four stored Q8_0 codes u = q + 128 -> two words of bf16 pairs (q0, q1), (q2, q3), exact: the low seven
-// bits in the mantissa of 128 (0x43xx) give 128 + (u & 127); 128 (u >= 128) or 256 (u < 128) off that is q.
-__device__ __forceinline__ void codes_q8(uint32_t w, uint32_t& p01, uint32_t& p23) {
-  const uint32_t lo = w & 0x7F7F7F7Fu, sb = ~w & 0x80808080u;
-  p01 = bf2_sub(__byte_perm(lo, 0x43434343u, 0x4140), __byte_perm(sb, 0x43434343u, 0x4140));
-  p23 = bf2_sub(__byte_perm(lo, 0x43434343u, 0x4342), __byte_perm(sb, 0x43434343u, 0x4342));
-}
-// Four 4-bit codes n in the bytes of w -> bf16 pairs of n - 8 (128 + n minus 136, exact)
-__device__ __forceinline__ void codes_q4(uint32_t w, uint32_t& p01, uint32_t& p23) {
-  p01 = bf2_sub(__byte_perm(w, 0x43434343u, 0x4140), 0x43084308u);
-  p23 = bf2_sub(__byte_perm(w, 0x43434343u, 0x4342), 0x43084308u);
 }
 
 // A fragments of one 32-weight block for the two K halves m = 0, 1 (k slots 2t, 2t + 1, 2t + 8, 2t + 9 of
