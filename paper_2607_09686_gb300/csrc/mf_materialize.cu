@@ -5,14 +5,16 @@
 //
 // The misses are decided on the device (slot resolve), so the copy is driven by the GPU
 // itself: SMs load 16-byte vectors straight from the pinned, device-mapped pack over the
-// CPU-GPU link and store them into the slot, with no host round trip.  Blocks stride over each
-// missed payload of the wave in turn (with no miss every block returns at once), 12 16-byte loads
-// in flight per thread.  A call of one wave has nothing beside the copy: a few large blocks on the
-// call's own stream.  In a call of several waves the copy runs on the context's side stream beside
-// the persistent expert kernels (one block per SM with a fixed share of the work): one block of 128
-// threads per SM, with at most 64 registers a thread, so that it fits beside a GEMM block (which has
-// all but 2048 registers of each SM sub-partition); 64 threads with 8 loads left the link idle
-// (4096 Q4_0 tokens on a cold 15 % cache: 2.92 ms a call, 2.59 ms this way).  The kernels here ask
+// CPU-GPU link and store them into the slot, with no host round trip.  The wave's missed
+// payloads are dealt to the blocks in chunks, 12 16-byte loads in flight per thread, so that every block
+// has copies in flight however small a payload is (one payload after another left most blocks idle: 35
+// misses of 418 KB took 393 us, 37 GB/s).  A call of one wave has nothing beside the copy: a few large
+// blocks on the call's own stream.  In a call of several waves the copy runs on the context's side
+// stream beside the persistent expert kernels (one block per SM with a fixed share of the work): one
+// block of 64 threads per SM, with at most 64 registers a thread, so that it fits beside a GEMM block
+// (which has all but 2048 registers of each SM sub-partition) or a streaming block.  4096 Q4_0 tokens
+// on a cold 15 % cache: 2.26 ms a call; 64 streams in waves: 1.31 ms (1.50 with 128 threads, of which
+// the streaming blocks leave no room for four warps).  The kernels here ask
 // for the largest shared-memory carveout although they use none: an SM runs blocks of one
 // carveout at a time, so only then can they share SMs with a running expert-FFN kernel (which
 // needs most of the shared memory) instead of holding those SMs until they finish.
@@ -26,7 +28,7 @@ namespace mf {
 namespace {
 
 constexpr int kUnroll = 12;
-constexpr int kMatThreadsSpread = 128;  // one block per SM
+constexpr int kMatThreadsSpread = 64;  // one block per SM
 constexpr int kMatThreadsDense = 512;  // one block per 8 SMs
 
 // dst_stage: null to write each miss into its slot, else miss m of the wave goes to
@@ -36,29 +38,27 @@ __global__ void __launch_bounds__(1024) k_materialize(Dev d, int layer, int wave
   pdl_trigger();
   pdl_wait();
   const int n_miss = d.info[2 + wave];
-  const uint32_t nvec = (uint32_t)(d.lay.stride / 16);  // 16-byte vectors per payload (32-bit: registers)
-  const uint32_t step = gridDim.x * blockDim.x * kUnroll;
+  const uint32_t nvec = (uint32_t)(d.lay.stride / 16);  // 16-byte vectors per payload
+  const uint32_t chunk = blockDim.x * kUnroll, per = (nvec + chunk - 1) / chunk;
 #pragma unroll 1
-  for (int m = 0; m < n_miss; ++m) {
+  for (uint32_t c = blockIdx.x; c < (uint32_t)n_miss * per; c += gridDim.x) {
+    const uint32_t m = c / per, i0 = (c - m * per) * chunk + threadIdx.x;
     const int u = d.miss_list[wave * d.S_active + m];
     const uint4* src = reinterpret_cast<const uint4*>(
         d.fstage ? d.fstage + (size_t)m * d.fstride  // a file-backed pack: the host staged miss m here
                  : d.pack + ((size_t)layer * d.E + d.uniq[u]) * d.lay.stride);
     uint4* dst = reinterpret_cast<uint4*>(dst_stage ? dst_stage + (size_t)m * d.lay.stride
                                                     : d.pool + ((size_t)layer * d.S_alloc + d.uslot[u]) * d.lay.stride);
-#pragma unroll 1
-    for (uint32_t i0 = blockIdx.x * blockDim.x * kUnroll + threadIdx.x; i0 < nvec; i0 += step) {
-      uint4 v[kUnroll];
+    uint4 v[kUnroll];
 #pragma unroll
-      for (int r = 0; r < kUnroll; ++r) {  // all loads first: kUnroll transfers in flight per thread
-        const uint32_t i = i0 + r * blockDim.x;
-        if (i < nvec) v[r] = ld_stream(src + i);
-      }
+    for (int r = 0; r < kUnroll; ++r) {  // all loads first: kUnroll transfers in flight per thread
+      const uint32_t i = i0 + r * blockDim.x;
+      if (i < nvec) v[r] = ld_stream(src + i);
+    }
 #pragma unroll
-      for (int r = 0; r < kUnroll; ++r) {
-        const uint32_t i = i0 + r * blockDim.x;
-        if (i < nvec) dst[i] = v[r];
-      }
+    for (int r = 0; r < kUnroll; ++r) {
+      const uint32_t i = i0 + r * blockDim.x;
+      if (i < nvec) dst[i] = v[r];
     }
   }
 }
