@@ -450,7 +450,36 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     s_xmax = kNoExp;
   }
   if (threadIdx.x < kMaxTopK) s_hmax[threadIdx.x] = kNoExp;
+  __syncthreads();  // the barriers are initialised
+  // The producer warp's first copies do not wait for the block's item list: where every expert is resident
+  // (the common case) item t is list position p = blockIdx.x + t * gridDim.x in rank order, so lane t knows
+  // its rank and row block before the router ends, and only the slots have to be read.
+  const int p_first = (int)blockIdx.x + lane * (int)gridDim.x, nrb0 = d.I / cg.R;
+  const int q_first = p_first / nrb0, rb_first = p_first - q_first * nrb0;
   pdl_wait();  // the router's outputs (and the caller's x) are complete and visible
+  int pre = 0;  // items (and then every down copy) already requested
+  if (warp == kConsumers && !d.hold) {
+    const int sl = lane < k ? d.uslot[lane] : 0, ms = lane < k ? d.umiss[lane] : 0;
+    if (!__ballot_sync(0xffffffffu, ms != 0)) {
+      pre = min(mine_g, min(f.NS, 32));
+      const uint64_t pol = l2_evict_first();
+      const uint8_t* pool0 = d.pool + (size_t)layer * d.S_alloc * d.lay.stride;
+      const int slot_q = __shfl_sync(0xffffffffu, sl, q_first & 31);
+      if (lane < pre) {
+        mbar_arrive_tx(&sm.full[lane], cg.stage_bytes);
+        bulk_g2s_hint(sm.stage0 + (size_t)lane * f.stage_bytes,
+                      pool0 + (size_t)slot_q * d.lay.stride + (size_t)rb_first * cg.R * d.lay.rs_gu, cg.stage_bytes,
+                      &sm.full[lane], pol);
+      }
+      if (lane < mine_d) {
+        const uint32_t dbytes = (uint32_t)nrows * d.lay.rs_d;
+        mbar_arrive_tx(&full_d[lane], dbytes);
+        bulk_g2s_hint(dbuf + (size_t)lane * f.dn_bytes,
+                      pool0 + (size_t)sl * d.lay.stride + d.lay.d_off + (size_t)r0 * d.lay.rs_d, dbytes, &full_d[lane], pol);
+      }
+    }
+    pre = __shfl_sync(0xffffffffu, pre, 0);
+  }
   // x split by kG = kW / 4 threads per group (consecutive lanes), each one word of four values,
   // where x has at most 512 words (H <= 2048); consumer thread t's word is requested while the
   // block sets up.  Larger x: one group per thread (split_vectors).
@@ -505,10 +534,11 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     const uint32_t dbytes = (uint32_t)nrows * d.lay.rs_d;
     const size_t doff = (size_t)r0 * d.lay.rs_d;
     const int n_issue = d.hold ? 0 : nres;
+    const bool all_hit = pre > 0 || (mine_g == 0 && NB == 0 && !d.hold);  // the first copies are under way
     // the resident experts' down records go after the first two gate/up items
     const int first = min(n_issue, min(2, NA));
     const uint64_t pol = l2_evict_first();  // read once per call: keep L2 for what is reused
-    bool d_issued = false;
+    bool d_issued = all_hit;
     auto issue_down_hits = [&]() {
       if (lane == 0)
         for (int j = 0; j < mine_d; ++j)
@@ -519,8 +549,14 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       d_issued = true;
     };
     if (lane == 0) {
-      for (int t = 0; t < n_issue; ++t, ++it) {
-        if (t == first) issue_down_hits();
+      it = pre;
+      if (pre == NA) {
+        ring.phase = 1;  // one round of the ring
+      } else {
+        ring.s = pre;
+      }
+      for (int t = pre; t < n_issue; ++t, ++it) {
+        if (t == first && !d_issued) issue_down_hits();
         if (it >= NA && !(ok = mbar_wait(&sm.empty[ring.s], ring.phase ^ 1u, d.wait_ns))) break;
         uint64_t* bar = &sm.full[ring.s];
         mbar_arrive_tx(bar, bytes);
