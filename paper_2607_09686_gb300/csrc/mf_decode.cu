@@ -86,24 +86,25 @@ __device__ __forceinline__ void split_vectors(const float* __restrict__ src, int
                                               int* s_max, int* s_exp) {
   constexpr int kW = Vec<QT>::kW;
   const int nt = kConsumers * 32, i0 = (int)threadIdx.x;
-  int eg[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = i0 + q * nt;
-    if (i < n) {
-      float v[kW];
-      load_group<QT, kCoherent>(src + (size_t)i * kW, v);
-      eg[q] = group_exponent(group_absmax<QT>(v));
-      dst[i] = quant_vals<QT>(v, eg[q] == kNoExp ? 0 : -eg[q]);
-      atomicMax(&s_max[i / per], eg[q]);
-    }
+  // (rolled loops: this code runs once per launch, and instructions that are fetched for it cost more
+  // than they compute -- a quarter of the kernel's stalls were instruction fetches)
+  int first = kNoExp, later[3] = {kNoExp, kNoExp, kNoExp};  // each group's exponent; seldom more than one a thread
+#pragma unroll 1
+  for (int i = i0, q = 0; i < n; i += nt, ++q) {
+    float v[kW];
+    load_group<QT, kCoherent>(src + (size_t)i * kW, v);
+    const int eg = group_exponent(group_absmax<QT>(v));
+    dst[i] = quant_vals<QT>(v, eg == kNoExp ? 0 : -eg);
+    if (q == 0)
+      first = eg;
+    else
+      later[q - 1] = eg;
+    atomicMax(&s_max[i / per], eg);
   }
   named_bar_sync(1, nt);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = i0 + q * nt;
-    if (i < n) rescale_group<QT>(dst[i], eg[q], vector_exponent(s_max[i / per]));
-  }
+#pragma unroll 1
+  for (int i = i0, q = 0; i < n; i += nt, ++q)
+    rescale_group<QT>(dst[i], q == 0 ? first : later[q - 1], vector_exponent(s_max[i / per]));
   for (int r = i0; r * per < n; r += nt) s_exp[r] = vector_exponent(s_max[r]);
   named_bar_sync(1, nt);
 }
@@ -400,11 +401,14 @@ struct FusedCfg {
 constexpr int kFusedBars = 2 * kMaxStages + kMaxTopK;
 
 // The arrival is a release (the block's h, written before it and published to this thread by the
-// block barrier, becomes visible with it); the polling loads acquire.  Bounded in time.
-__device__ __forceinline__ bool grid_arrive_wait(unsigned long long* arrive, unsigned* err, uint64_t limit_ns) {
-  unsigned long long old;
-  asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(arrive) : "memory");
-  const unsigned long long target = (old / gridDim.x + 1) * gridDim.x;
+// block barrier, becomes visible with it); the polling loads acquire.  `seen` is the counter as read
+// before this block's arrival: every earlier launch is complete and this one cannot complete without this
+// block, so the next multiple of gridDim.x is the one to wait for, and the addition need not return.
+// Bounded in time.
+__device__ __forceinline__ bool grid_arrive_wait(unsigned long long* arrive, unsigned long long seen, unsigned* err,
+                                                 uint64_t limit_ns) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(arrive) : "memory");
+  const unsigned long long target = (seen / gridDim.x + 1) * gridDim.x;
   if (counter_wait(arrive, target, limit_ns)) return true;
   atomicExch(err, 5u);
   return false;
@@ -488,23 +492,73 @@ __global__ void __launch_bounds__(kThreadsF, 1)
   const bool x_mine = x_words && warp < kConsumers && (int)threadIdx.x < cg.n_vec * kG;
   float4 xv = make_float4(0.f, 0.f, 0.f, 0.f);
   if (x_mine) xv = __ldg(reinterpret_cast<const float4*>(x) + threadIdx.x);
-  if (threadIdx.x < k) {  // one token: access u = rank j
-    uint8_t* slot = d.pool + ((size_t)layer * d.S_alloc + d.uslot[threadIdx.x]) * d.lay.stride;
-    s_gu[threadIdx.x] = slot;
-    s_dn[threadIdx.x] = slot + d.lay.d_off;
-    s_hgu[threadIdx.x] = d.fstage ? d.fstage + (size_t)threadIdx.x * d.fstride  // staged from the file
-                                  : d.pack + ((size_t)layer * d.E + d.uniq[threadIdx.x]) * d.lay.stride;
-    s_g[threadIdx.x] = d.g[threadIdx.x];
-    s_miss[threadIdx.x] = d.umiss[threadIdx.x];
-  }
-  __syncthreads();
-  if (warp == 0) {
+  auto split_x = [&]() {  // the consumers
+    if (x_words) {  // x split into int8 pieces, scaled by the power of two of its largest magnitude:
+                    // the same pieces as quant_vals of the whole group (the group's largest
+                    // magnitude m by shuffles, each value scaled by 2^-e_g and split by
+                    // 127 / (m 2^-e_g), the piece sums added over the kG threads), then the
+                    // vector's exponent and rescale_group as in split_vectors
+      XQ<QT>* dst = reinterpret_cast<XQ<QT>*>(sm.vq);
+      const int gi = threadIdx.x / kG, part = threadIdx.x % kG;
+      float m = fmaxf(fmaxf(fabsf(xv.x), fabsf(xv.y)), fmaxf(fabsf(xv.z), fabsf(xv.w)));
+#pragma unroll
+      for (int o = 1; o < kG; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      const int eg = group_exponent(m), ne = eg == kNoExp ? 0 : -eg;
+      const float sa = pow2i(ne / 2), sb = pow2i(ne - ne / 2);
+      const float ms = m * sa * sb;  // exact: the largest value scaled by a power of two
+      const float inv = ms > 0x1p-100f ? 127.f / ms : 0.f;
+      const float vv[4] = {xv.x * sa * sb, xv.y * sa * sb, xv.z * sa * sb, xv.w * sa * sb};
+      uint32_t b1, b2, b3;
+      const float tt[4] = {__fmul_rn(vv[0], inv), __fmul_rn(vv[1], inv), __fmul_rn(vv[2], inv), __fmul_rn(vv[3], inv)};
+      quant4(tt, b1, b2, b3);
+      int s1 = byte_sum(b1, 0), s2 = byte_sum(b2, 0), s3 = byte_sum(b3, 0);
+#pragma unroll
+      for (int o = 1; o < kG; o <<= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        s3 += __shfl_xor_sync(0xffffffffu, s3, o);
+      }
+      if (x_mine) {
+        dst[gi].p1[part] = b1;
+        dst[gi].p2[part] = b2;
+        dst[gi].p3[part] = b3;
+        if (part == 0) {
+          constexpr int off = QT == kQ8 ? 128 : 8;
+          dst[gi].k12 = off * (s1 * 127 + s2);
+          dst[gi].k3 = off * s3;
+          dst[gi].sf = inv > 0.f ? ms / 127.f / 16129.f : 0.f;
+          atomicMax(&s_xmax, eg);
+        }
+      }
+      named_bar_sync(1, kConsumers * 32);
+      if (x_mine && part == 0) rescale_group<QT>(dst[gi], eg, vector_exponent(s_xmax));
+      if (threadIdx.x == 0) s_xexp = vector_exponent(s_xmax);
+      named_bar_sync(1, kConsumers * 32);
+    } else {
+      split_vectors<QT>(x, cg.n_vec, cg.n_vec, reinterpret_cast<XQ<QT>*>(sm.vq), &s_xmax, &s_xexp);
+    }
+  };
+  unsigned long long seen = 0;
+  if (threadIdx.x == 0) seen = *reinterpret_cast<volatile unsigned long long*>(d.work);
+  if (warp == kConsumers + 1) {
+    // the link warp reads the routing outputs and forms the item list while the consumers split x
+    int ms = 0;
+    if (lane < k) {  // one token: access u = rank j
+      uint8_t* slot = d.pool + ((size_t)layer * d.S_alloc + d.uslot[lane]) * d.lay.stride;
+      s_gu[lane] = slot;
+      s_dn[lane] = slot + d.lay.d_off;
+      s_hgu[lane] = d.fstage ? d.fstage + (size_t)lane * d.fstride  // staged from the file
+                             : d.pack + ((size_t)layer * d.E + d.uniq[lane]) * d.lay.stride;
+      s_g[lane] = d.g[lane];
+      s_miss[lane] = ms = d.umiss[lane];
+    }
+    __syncwarp();
     // list position p = blockIdx.x + t * gridDim.x (lane t); the list holds the resident experts'
     // items, then the missed experts' (ranks in order within each); item id = rank * (I / R) + row
     // block.  Position q of the expert list: the q-th resident rank, or the (q - n_res)-th missed one.
     const int nrb = d.I / cg.R;
     const unsigned kmask = (1u << k) - 1u;
-    const unsigned res = __ballot_sync(0xffffffffu, lane < k && !s_miss[lane]);
+    const unsigned res = __ballot_sync(0xffffffffu, lane < k && !ms);
     const int n_res_e = __popc(res);
     for (int t = lane; t < mine_g; t += 32) {
       const int p = (int)blockIdx.x + t * (int)gridDim.x, q = p / nrb;
@@ -519,6 +573,8 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       s_nres = lim <= 0 ? 0 : min(mine_g, (lim + (int)gridDim.x - 1) / (int)gridDim.x);
       s_nb = n_res_e < k ? 2 : 0;  // ring B only when the call has a missed expert (NS >= 4)
     }
+  } else if (warp < kConsumers) {
+    split_x();
   }
   __syncthreads();
 
@@ -646,62 +702,6 @@ __global__ void __launch_bounds__(kThreadsF, 1)
       const int nv = (d.lay.qrow_gu / 16) / cs;
       const int v0 = col * nv;
       const XQ<QT>* xq = reinterpret_cast<const XQ<QT>*>(sm.vq);
-      if (x_words) {  // x split into int8 pieces, scaled by the power of two of its largest magnitude:
-                      // the same pieces as quant_vals of the whole group (the group's largest
-                      // magnitude m by shuffles, each value scaled by 2^-e_g and split by
-                      // 127 / (m 2^-e_g), the piece sums added over the kG threads), then the
-                      // vector's exponent and rescale_group as in split_vectors
-        XQ<QT>* dst = reinterpret_cast<XQ<QT>*>(sm.vq);
-        const int gi = threadIdx.x / kG, part = threadIdx.x % kG;
-        float m = fmaxf(fmaxf(fabsf(xv.x), fabsf(xv.y)), fmaxf(fabsf(xv.z), fabsf(xv.w)));
-#pragma unroll
-        for (int o = 1; o < kG; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const int eg = group_exponent(m), ne = eg == kNoExp ? 0 : -eg;
-        const float sa = pow2i(ne / 2), sb = pow2i(ne - ne / 2);
-        const float ms = m * sa * sb;  // exact: the largest value scaled by a power of two
-        const float inv = ms > 0x1p-100f ? 127.f / ms : 0.f;
-        const float vv[4] = {xv.x * sa * sb, xv.y * sa * sb, xv.z * sa * sb, xv.w * sa * sb};
-        uint32_t b1 = 0, b2 = 0, b3 = 0;
-        int s1 = 0, s2 = 0, s3 = 0;
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-          const float t = vv[jj] * inv;
-          const int a = __float2int_rn(t);
-          const float e = (t - (float)a) * 127.f;
-          const int b = __float2int_rn(e);
-          const int c = __float2int_rn((e - (float)b) * 127.f);
-          s1 += a;
-          s2 += b;
-          s3 += c;
-          b1 |= (uint32_t)(a & 0xFF) << (8 * jj);
-          b2 |= (uint32_t)(b & 0xFF) << (8 * jj);
-          b3 |= (uint32_t)(c & 0xFF) << (8 * jj);
-        }
-#pragma unroll
-        for (int o = 1; o < kG; o <<= 1) {
-          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-          s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-        }
-        if (x_mine) {
-          dst[gi].p1[part] = b1;
-          dst[gi].p2[part] = b2;
-          dst[gi].p3[part] = b3;
-          if (part == 0) {
-            constexpr int off = QT == kQ8 ? 128 : 8;
-            dst[gi].k12 = off * (s1 * 127 + s2);
-            dst[gi].k3 = off * s3;
-            dst[gi].sf = inv > 0.f ? ms / 127.f / 16129.f : 0.f;
-            atomicMax(&s_xmax, eg);
-          }
-        }
-        named_bar_sync(1, kConsumers * 32);
-        if (x_mine && part == 0) rescale_group<QT>(dst[gi], eg, vector_exponent(s_xmax));
-        if (threadIdx.x == 0) s_xexp = vector_exponent(s_xmax);
-        named_bar_sync(1, kConsumers * 32);
-      } else {
-        split_vectors<QT>(x, cg.n_vec, cg.n_vec, reinterpret_cast<XQ<QT>*>(sm.vq), &s_xmax, &s_xexp);
-      }
       XQ<QT> xr[VPL];
 #pragma unroll
       for (int i = 0; i < VPL; ++i) {
@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(kThreadsF, 1)
     }
     if (!ok && lane == 0) atomicExch(d.err, 3u);
     // ---- every block's h published (one arrival per block, always, so launches stay aligned)
-    if (threadIdx.x == 0 && !grid_arrive_wait(d.work, d.err, d.wait_ns)) ok = false;
+    if (threadIdx.x == 0 && !grid_arrive_wait(d.work, seen, d.err, d.wait_ns)) ok = false;
     named_bar_sync(1, kConsumers * 32);
     // ---- down: warp w holds expert j = w / (16 / k)'s h in registers for the whole phase and
     // takes rows sub, sub + 16 / k, ... of that expert's item (sub = w % (16 / k))
