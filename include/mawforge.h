@@ -14,7 +14,8 @@
  * mf_moe_forward runs, for one layer and T tokens, entirely in CUDA kernels:
  *   router logits + top-k + softmax over the chosen ->
  *   slot resolve (per-layer LRU, hit / miss / eviction / byte counters) ->
- *   materialisation of the missed payloads, pinned host -> HBM slot, on a side stream ->
+ *   materialisation of the missed payloads, pinned host -> HBM slot (in a call of several waves
+ *     on a side stream, beside the expert kernels) ->
  *   dequantising gate/up projections + SwiGLU -> down projection + router-weighted combine.
  *
  * Conventions for every entry point:
@@ -220,8 +221,9 @@ int mf_moe_forward(mf_ctx_t* ctx, int layer, const float* x, const float* router
  * GEMMs (section "Native Serving Path"'s expert FFN, batched over the tokens each expert
  * serves, as for a prefill chunk): per (expert, 128 assignments, 128 weight rows) the
  * dequantised Q8_0 / Q4_0 weights and the activations, each split into bf16 hi + lo, are
- * multiplied on the tensor cores with fp32 accumulation (hi*hi + hi*lo + lo*hi).  Smaller T
- * use the dequantising GEMV kernels.  The default is 256 when the plan's max_tokens >= 256,
+ * multiplied on the tensor cores with fp32 accumulation (hi*hi + hi*lo + lo*hi).  Smaller
+ * T > 1 stream each expert's codes through warp-level MMAs with the activations in three exact
+ * bf16 pieces (fp32 accuracy); T = 1 uses the dequantising GEMV kernels.  The default is 256 when the plan's max_tokens >= 256,
  * else 0 (off).  min_tokens = 0 disables the GEMM path; otherwise it must be >= 2, the plan's
  * max_tokens >= 2 and hidden and inter multiples of 128 (MF_E_INVAL otherwise).  Enabling it
  * on a context created with max_tokens < 256 allocates its operand tiles here:

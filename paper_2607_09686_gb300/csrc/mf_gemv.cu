@@ -1,4 +1,4 @@
-// Decode expert FFN: dequantising GEMV over the experts resident in HBM slots.
+// One-token expert FFN, general shapes: dequantising GEMV over the experts resident in HBM slots.
 //
 //   h[t,j][r] = silu(sum_c Wg_e[r,c] x_t[c]) * sum_c Wu_e[r,c] x_t[c]     (gate/up + SwiGLU)
 //   y[t][c]   = sum_j g[t,j] * sum_r Wd_e[c,r] h[t,j][r]                  (down + combine)
@@ -11,8 +11,7 @@
 //
 // One warp per weight row.  Each lane holds whole 16-byte vectors of the row's codes in
 // registers (Q8_0: 16 weights, Q4_0: one 32-weight block).  Codes are turned into floats exactly by
-// placing each byte (or
-// nibble) in the low mantissa bits of 2^23 with a byte permute and subtracting 2^23 plus
+// placing each byte (or nibble) in the low mantissa bits of 2^23 with a byte permute and subtracting 2^23 plus
 // the code offset (the int8 -> float "magic number" conversion of Kim et al., "Who says
 // elephants can't run", 2022), which costs one PRMT and one FADD per weight instead of an
 // integer-to-float conversion.  The scale multiplies each vector's partial dot product.
