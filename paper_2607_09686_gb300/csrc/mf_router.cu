@@ -23,6 +23,8 @@
 // singles out the experts that can be chosen, and compute those exactly: see k_logits_fp32.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "mf_lru.cuh"
 
 namespace cg = cooperative_groups;
@@ -291,7 +293,9 @@ __global__ void __launch_bounds__(kThreadsR)
 // logit as a plain fp32 dot product (one FMA per product instead of Dot2's ten operations), k_topk_exact
 // bounds each one's error, keeps the experts whose bound reaches the k-th largest logit, and computes
 // those (k and the rare close call) with the compensated dot product, which alone decides: the routing
-// and the weights are those of exact logits for every expert.
+// and the weights are those of exact logits for every expert.  Bound: fp32 issue of the plain product (4096
+// tokens, 128 experts, hidden 2048: 79 us), then the exact ones' re-reading of k rows of W_r per token (80
+// us); compensated dot products for every expert took 385 + 31 us there.
 //
 // k_logits_fp32: block (expert tile, token tile, K split) computes a 64-token x 16 J-expert tile over its
 // range of H, from shared-memory tiles of x and W_r that cp.async fills 16 columns at a time
@@ -544,19 +548,24 @@ __global__ void __launch_bounds__(kThreadsTop, 4)
   if (warp == 0) softmax_topk(d, t, k, s_sel, s_zs);
 }
 
-// K splits for T tokens: about kTiledBlocks blocks when the tiles alone are fewer.  A constant
-// (two blocks per SM of a 152-SM part), not the device's count, so that the planner, which runs
-// without a GPU, sizes the scratch exactly as the context does.
-constexpr int kTiledBlocks = 304, kMaxSplits = 64;
+// K splits for T tokens.  At least about kTiledBlocks blocks (two per SM) when the tiles alone are fewer;
+// from there to twice as many splits, the number whose busiest SM walks the fewest chunks: 64 token tiles
+// (4096 tokens) in 5 splits left 16 of 320 blocks to a round of their own, in 7 the call is 17 us shorter.
+// Constants (of a 152-SM part), not the device's count, so that the planner, which runs without a GPU,
+// sizes the scratch exactly as the context does.
+constexpr int kTiledSms = 152, kTiledBlocks = 2 * kTiledSms, kMaxSplits = 64;
 int tile_experts(int E) { return E > 64 ? 128 : 64; }
 int tiled_splits(int T, int E, int H) {
   const int tiles = ((T + kTT - 1) / kTT) * ((E + tile_experts(E) - 1) / tile_experts(E));
   const int nch = H / kHC;
-  int want = (kTiledBlocks + tiles - 1) / tiles;
-  if (want < 1) want = 1;
-  if (want > kMaxSplits) want = kMaxSplits;
-  const int cps = (nch + want - 1) / want;
-  return (nch + cps - 1) / cps;
+  const int want = std::min(kMaxSplits, std::max(1, (kTiledBlocks + tiles - 1) / tiles));
+  int best = 0, best_cost = 0;
+  for (int w = want; w <= std::min(kMaxSplits, 2 * want); ++w) {
+    const int cps = (nch + w - 1) / w, ks = (nch + cps - 1) / cps;
+    const int cost = (tiles * ks + kTiledSms - 1) / kTiledSms * cps;
+    if (best == 0 || cost < best_cost) best = ks, best_cost = cost;
+  }
+  return best;
 }
 
 cudaError_t launch_router_tiled(const Dev& d, const float* x, const float* wr, const float* bias, int T,
@@ -580,7 +589,9 @@ cudaError_t launch_router_tiled(const Dev& d, const float* x, const float* wr, c
 
 size_t router_part_floats(int T_max, int E, int H) {
   size_t most = 0;
-  for (int T = kTiledMinT; T <= T_max; ++T) {
+  for (int t0 = 0; t0 < T_max; t0 += kTT) {  // the splits depend on the number of token tiles only
+    const int T = std::min(t0 + kTT, T_max);
+    if (T < kTiledMinT) continue;
     const size_t n = (size_t)tiled_splits(T, E, H) * ((size_t)T + 1) * E;
     if (n > most) most = n;
   }
