@@ -37,7 +37,10 @@
 //                        lanes, half of the columns each); the next unit's MMAs wait for that, the
 //                        converters and copies run ahead.
 // Tensor memory: 256 columns of accumulators, 4 A stages of 64 columns.  What bounds it: the MMAs
-// (three products per weight).  With A in shared memory the MMAs' operand reads, the converters'
+// (three products per weight: 768 cycles of a step's 1200 at 128 assignments) and, between two units, the
+// epilogue's reading of the one accumulator set there is room for (150-280 cycles a step).  4096 tokens,
+// 128 Q4_0 experts of 2048 x 768: gate/up 444 us and down 293 us, where units of 128 rows with A in shared
+// memory took 638 and 446.  With A in shared memory the MMAs' operand reads, the converters'
 // stores and the B copies together filled the shared-memory pipe (an M = 128, N = 128, K = 16 MMA
 // reads 8 KiB of it per 64 tensor cycles; down units of 128 rows also loaded a B tile per 128 rows).
 // Every wait is bounded; a wait that gives up sets the block's flag and the device error word,
@@ -590,7 +593,11 @@ __global__ void __launch_bounds__(1024, 1)
 
 // x (fp32 [T][H]) -> the x tiles of every 128-assignment block of the call: block t (of unique
 // expert u, assignments asg_off[u] + 128 tb ..), K step kk: column c = assignment, row k,
-// split into bf16 hi and lo; columns past the expert's assignments are zero.
+// split into bf16 hi and lo; columns past the expert's assignments, up to the next multiple of 16, are zero.
+// Bound: HBM (4 bytes written per assignment and weight column; the rows are re-read from L2), given enough
+// blocks: a tile's K steps are dealt to as many blocks as keep the launch at about six per SM (one per tile
+// was two or three per SM: 1000 tokens 357 -> 319 us a call, 4096 1067 -> 1050).  Eight fill an SM's threads,
+// and the materialiser running beside them then waits for its place (4096 tokens with misses: 2.25 -> 2.29 ms).
 __global__ void __launch_bounds__(256) k_tile_x(Dev d, const float* __restrict__ x) {
   __shared__ int s_row[kBN];
   __shared__ int s_u, s_tb;
@@ -611,11 +618,13 @@ __global__ void __launch_bounds__(256) k_tile_x(Dev d, const float* __restrict__
   const int a0 = d.asg_off[s_u] + s_tb * kBN, n = min(kBN, d.asg_off[s_u + 1] - a0);
   for (int c = threadIdx.x; c < kBN; c += blockDim.x) s_row[c] = c < n ? d.asg[a0 + c] / d.k : -1;
   __syncthreads();
-  const int nk = d.H / kBK;
-  uint8_t* tile0 = d.xt + (size_t)t * nk * kBTile;
+  const int steps = d.H / kBK;
+  uint8_t* tile0 = d.xt + (size_t)t * steps * kBTile;
+  // K steps [k0, nk): this block's share of the tile
+  const int k0 = steps * (int)blockIdx.y / (int)gridDim.y, nk = steps * ((int)blockIdx.y + 1) / (int)gridDim.y;
   // item i = (column i >> 2, 8-value group i & 3) of one K step
   const int per = n_eff(n) * 4;  // items of a K step: the columns the MMAs read
-  int kk = threadIdx.x / per, i = threadIdx.x % per;
+  int kk = k0 + threadIdx.x / per, i = threadIdx.x % per;
   for (; kk < nk; i += blockDim.x) {
     while (i >= per) i -= per, ++kk;
     if (kk >= nk) break;
@@ -711,7 +720,9 @@ int prefill_tensor_maps(mf_ctx* c) {
 
 cudaError_t launch_tile_x(const Dev& d, const float* x, int T, cudaStream_t s) {
   const uint64_t blocks = prefill_tiles_max(T, d.k, d.E);
-  k_tile_x<<<(unsigned)blocks, 256, 0, s>>>(d, x);
+  const uint64_t most = (uint64_t)d.H / kBK, room = 6 * (uint64_t)sm_count_p() / blocks;
+  const uint64_t split = room < 1 ? 1 : room > most ? most : room;
+  k_tile_x<<<dim3((unsigned)blocks, (unsigned)split), 256, 0, s>>>(d, x);
   return cudaGetLastError();
 }
 
