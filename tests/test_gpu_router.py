@@ -110,3 +110,33 @@ def test_tiled_router_orders_logits_that_fp32_sums_cannot(E, T):
         _check_routes(ctx, synth.activations(23, 0, 0, 0, T, H), None, T, k)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("T", [1, 5, 20])
+def test_indices_and_weights_reach_any_buffer(T, off):
+    """The router stores idx and w itself where the caller's buffers are aligned to their values; buffers
+    at an odd address (off = 1) are copied to.  Either one alone, and neighbouring bytes left as they were."""
+    H, E, k = 256, 40, 5
+    shape = Shape(1, H, E, k, 64, synth.Q8_0, model_seed=10)
+    ctx = Ctx(shape, slots=E, max_tokens=T)
+    try:
+        torch, n = ctx.torch, T * k * 4
+        xh = synth.activations(24, 0, 0, 0, T, H)
+        x, y = torch.from_numpy(xh).to(ctx.device), torch.empty(T, H, device=ctx.device)
+        for want_i, want_w in ((True, True), (True, False), (False, True)):
+            bufs = [torch.full((n + 16,), 0xA5, dtype=torch.uint8, device=ctx.device) for _ in range(2)]
+            at = [b.data_ptr() + off if want else None for b, want in zip(bufs, (want_i, want_w))]
+            ctx.mf.mf_moe_forward(ctx.h, 0, x, ctx.wr[0], None, T, y, at[0], at[1])
+            torch.cuda.synchronize()
+            raw = [b.cpu().numpy() for b in bufs]
+            for r, want in zip(raw, (want_i, want_w)):
+                assert (r[:off] == 0xA5).all() and (r[off + n if want else 0:] == 0xA5).all()
+            idx = raw[0][off:off + n].copy().view(np.int32).reshape(T, k)
+            w = raw[1][off:off + n].copy().view(np.float32).reshape(T, k)
+            for t in range(T):
+                _, oidx, og = oracle.router(xh[t], ctx.wr_host[0], None, k)
+                assert not want_i or np.array_equal(idx[t], oidx), t
+                assert not want_w or np.abs(w[t] - og).max() <= G_ATOL, t
+    finally:
+        ctx.close()
