@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kThreadsR)
 // bounds each one's error, keeps the experts whose bound reaches the k-th largest logit, and computes
 // those (k and the rare close call) with the compensated dot product, which alone decides: the routing
 // and the weights are those of exact logits for every expert.  Bound: fp32 issue of the plain product (4096
-// tokens, 128 experts, hidden 2048: 79 us), then the exact ones' re-reading of k rows of W_r per token (80
+// tokens, 128 experts, hidden 2048: 62 us), then the exact ones' re-reading of k rows of W_r per token (80
 // us); compensated dot products for every expert took 385 + 31 us there.
 //
 // k_logits_fp32: block (expert tile, token tile, K split) computes a 64-token x 16 J-expert tile over its
