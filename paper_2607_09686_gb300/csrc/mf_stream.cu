@@ -72,14 +72,15 @@ struct SL {  // shared-memory stage: codes of two boxes, their scales, the activ
 };
 
 struct StreamCfg {
-  int NS, cols;          // stages; most assignments a unit of this call holds (a multiple of 8)
+  int NS, cols;          // stages; assignments per unit (a multiple of 8, at most kSCols): no unit holds more,
+                         // whatever the routes are, as a stage and the exchange buffers have room for these
   uint32_t stage;        // bytes per stage (a multiple of 1024)
   uint32_t off_bar, off_red, off_tab, total;
 };
 
 StreamCfg stream_cfg(const Dev& d, int T) {
   StreamCfg c;
-  c.cols = T >= kSCols ? kSCols : (T + 7) & ~7;  // a token takes an expert at most once
+  c.cols = T >= kSCols ? kSCols : (T + 7) & ~7;  // one unit per row block: a token takes an expert at most once
   const uint32_t a = d.qtype == MF_Q8_0 ? SL<kQ8>::kOffB : SL<kQ4>::kOffB;
   c.stage = (a + (uint32_t)c.cols * kColStride + 1023) & ~1023u;
   const uint32_t red = 2u * 8 * 32 * (c.cols / 8) * 16;  // two buffers of the K halves' sums
@@ -317,11 +318,11 @@ __global__ void __launch_bounds__(kSThreads, 1)
     if (i < nu) s_slot[i] = d.uslot[u0 + i];
   }
   __syncthreads();
-  if (warp == 0) {  // units before expert i: row blocks x groups of up to 32 assignments
+  if (warp == 0) {  // units before expert i: row blocks x groups of up to f.cols assignments
     int base = 0;
     for (int i0 = 0; i0 < nu; i0 += 32) {
       const int i = i0 + lane;
-      int v = i < nu ? (s_asg[i + 1] - s_asg[i] + kSCols - 1) / kSCols * nrb : 0;
+      int v = i < nu ? (s_asg[i + 1] - s_asg[i] + f.cols - 1) / f.cols * nrb : 0;
       const int own = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -342,8 +343,8 @@ __global__ void __launch_bounds__(kSThreads, 1)
       if (s_units[mid] <= i) lo = mid;
       else hi = mid - 1;
     }
-    const int r = i - s_units[lo], cb = r / nrb, n = s_asg[lo + 1] - s_asg[lo] - cb * kSCols;
-    return {layer * d.S_alloc + s_slot[lo], (r - cb * nrb) * kUnitRows, s_asg[lo] + cb * kSCols, min(n, kSCols)};
+    const int r = i - s_units[lo], cb = r / nrb, n = s_asg[lo + 1] - s_asg[lo] - cb * f.cols;
+    return {layer * d.S_alloc + s_slot[lo], (r - cb * nrb) * kUnitRows, s_asg[lo] + cb * f.cols, min(n, f.cols)};
   };
 
   if (warp == kSWarps) {  // ---- producer warp

@@ -38,3 +38,33 @@ def test_stream_tile_edges(qtype, H, I):
         assert ctx.mf.mf_check(ctx.h) == 0
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("E,k,slots", [(8, 8, 8), (12, 3, 12), (12, 3, 3)])
+@pytest.mark.parametrize("T", [5, 8, 16, 24])
+def test_tokens_whose_logits_overflow_leave_the_others_alone(E, k, slots, T):
+    """Finite inputs whose router products overflow give logits that are not numbers, and a choice of
+    experts that means nothing: the other tokens of the call keep their outputs, and every chosen index is
+    an expert.  A stage of the streaming kernels has room for T rounded up to 8 assignments, whatever the
+    choice is."""
+    H, I = 64, 96
+    shape = Shape(1, H, E, k, I, synth.Q8_0, model_seed=11)
+    ctx = Ctx(shape, slots, max_tokens=T)
+    pays = Payloads(shape)
+    try:
+        wr = ctx.wr_host[0].copy()
+        wr[:, 0] = 4.0
+        ctx.wr_host[0] = wr
+        ctx.wr[0] = ctx.torch.from_numpy(wr).to(ctx.device)
+        x = synth.activations(31, 0, 0, 0, T, H)
+        x[:, 0] = 0.0
+        good = np.arange(T) % 3 == 1
+        x[~good, 0] = 3e38
+        y, idx, _ = ctx.forward(0, x, None, T)
+        assert ((idx >= 0) & (idx < E)).all()
+        yo, io, _ = oracle.layer(pays.for_layer(0, range(E)), synth.Q8_0, H, I, k, wr, None, x[good])
+        assert np.array_equal(idx[good], io)
+        assert_outputs_close(y[good], yo, f"T {T}")
+        assert ctx.mf.mf_check(ctx.h) == 0
+    finally:
+        ctx.close()
