@@ -118,9 +118,13 @@ __device__ __forceinline__ bool cluster_rank_zero() {
   return r == 0;
 }
 
+// The logit by which an expert is ranked: one that is not a number counts as the lowest, so that the order
+// is total and the k first places name k distinct experts whatever the inputs are.
+__device__ __forceinline__ float rank_key(float z) { return fmaxf(z, -INFINITY); }
+
 // Rank by counting: position of expert e = experts with a larger logit, or equal and lower id; the k
 // first to s_sel / s_zsel.  tpe consecutive lanes share an expert, each counting over every tpe-th other
-// expert.  The block's z and s_sel are written before (with a barrier); ends with a barrier.
+// expert.  The block's z are written before (with a barrier); ends with a barrier.
 template <int kThreads>
 __device__ __forceinline__ void rank_topk(const float* s_z, int E, int k, int* s_sel, float* s_zsel) {
   const int tid = threadIdx.x;
@@ -130,17 +134,17 @@ __device__ __forceinline__ void rank_topk(const float* s_z, int E, int k, int* s
   for (int e0 = 0; e0 < E; e0 += per_pass) {  // block-uniform
     const int e = e0 + tid / tpe;
     const bool valid = e < E;
-    const float z = valid ? s_z[e] : 0.f;
+    const float z = valid ? rank_key(s_z[e]) : 0.f;
     int r = 0;
     if (valid)
       for (int e2 = part; e2 < E; e2 += tpe) {
-        const float z2 = s_z[e2];
+        const float z2 = rank_key(s_z[e2]);
         r += (z2 > z) || (z2 == z && e2 < e);
       }
     for (int off = tpe >> 1; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
     if (valid && part == 0 && r < k) {
       s_sel[r] = e;
-      s_zsel[r] = z;
+      s_zsel[r] = s_z[e];
     }
   }
   __syncthreads();
@@ -259,8 +263,6 @@ __global__ void __launch_bounds__(kThreadsR)
   if (rank != 0) return;
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-  if (tid < k) s_sel[tid] = tid;  // a valid choice even where the logits are not ordered (NaN)
-  __syncthreads();
   rank_topk<kThreadsR>(s_z, E, k, s_sel, s_zsel);
   if (warp == 0) softmax_topk(d, t, k, s_sel, s_zsel);
   if (!resolve) return;
@@ -437,7 +439,6 @@ __global__ void __launch_bounds__(kThreadsTop, 4)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) nx += __shfl_xor_sync(0xffffffffu, nx, o);
   if (lane == 0) s_n[warp] = nx;
-  if (tid < k) s_sel[tid] = tid;  // valid even where the logits are not ordered (NaN)
   if (tid == 0) s_nc = s_all = 0;
   __syncthreads();
   nx = 0.f;
@@ -535,13 +536,16 @@ __global__ void __launch_bounds__(kThreadsTop, 4)
   }
   __syncthreads();
   for (int c = tid; c < nc; c += kThreadsTop) {  // rank the candidates, ties to the lower id
-    const float z = s_a[c];
+    const float z = rank_key(s_a[c]);
     const int e = s_cand[c];
     int r = 0;
-    for (int c2 = 0; c2 < nc; ++c2) r += (s_a[c2] > z) || (s_a[c2] == z && s_cand[c2] < e);
+    for (int c2 = 0; c2 < nc; ++c2) {
+      const float z2 = rank_key(s_a[c2]);
+      r += (z2 > z) || (z2 == z && s_cand[c2] < e);
+    }
     if (r < k) {
       s_sel[r] = e;
-      s_zs[r] = z;
+      s_zs[r] = s_a[c];
     }
   }
   __syncthreads();

@@ -140,3 +140,36 @@ def test_indices_and_weights_reach_any_buffer(T, off):
                 assert not want_w or np.abs(w[t] - og).max() <= G_ATOL, t
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("E,k,n_nan", [(40, 5, 40), (40, 5, 38), (8, 8, 3), (200, 8, 200)])
+@pytest.mark.parametrize("T", [1, 5, 20])
+def test_logits_that_are_not_numbers_rank_last(T, E, k, n_nan):
+    """Finite inputs whose products overflow (x[0] times four of column 0) give logits that are not
+    numbers: they rank after every other, among themselves the lower expert first, so a token's k experts
+    are distinct and the same on every call; tokens with x[0] = 0 route as the oracle says."""
+    H = 256
+    shape = Shape(1, H, E, k, 64, synth.Q8_0, model_seed=12)
+    ctx = Ctx(shape, slots=E, max_tokens=T)
+    try:
+        bad = np.sort(np.random.default_rng(E + k).permutation(E)[:n_nan])
+        fine = np.setdiff1d(np.arange(E), bad)
+        wr = ctx.wr_host[0].copy()
+        wr[:, 0] = 0.0
+        wr[bad, 0] = 4.0
+        ctx.wr_host[0] = wr
+        ctx.wr[0] = ctx.torch.from_numpy(wr).to(ctx.device)
+        x = synth.activations(25, 0, 0, 0, T, H)
+        x[:, 0] = 0.0
+        x[::2, 0] = 3e38
+        _, idx, w = ctx.forward(0, x, None, T)
+        for t in range(T):
+            if t % 2 == 0:
+                z = wr[fine].astype(np.float64) @ x[t].astype(np.float64)
+                order = fine[np.lexsort((fine, -z.astype(np.float32)))]
+                assert np.array_equal(idx[t], np.concatenate([order, bad])[:k]), t
+            else:
+                _, oidx, og = oracle.router(x[t], wr, None, k)
+                assert np.array_equal(idx[t], oidx) and np.abs(w[t] - og).max() <= G_ATOL, t
+    finally:
+        ctx.close()
