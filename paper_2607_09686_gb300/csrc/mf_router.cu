@@ -409,6 +409,8 @@ constexpr int kThreadsTop = 256;
 // in flight).  Then, with a the fp32 logit and |a - exact| <= B:
 //   a sum of H products in two chains, added over the splits, is off by less than
 //   (H / 2 + splits + 8) 2^-24 sum |x w| <= (H + 64) 2^-24 |x|_2 |w|_2 and H 2^-148 where products underflow;
+//   a squared norm summed in fp32 may be short by 2^-150 for each of its H terms where squares underflow
+//   (values below 2^-63 or so), and is taken H 2^-149 longer;
 //   2^-21 of the logit's and the bias's magnitude covers the roundings after it (to fp32, the bias added).
 // L = the k-th largest of a - B is at or below the k-th largest exact logit, so an expert with a + B < L is
 // not chosen, not even on a tie.  The others are computed exactly, one warp each.  A bound that is not a
@@ -445,7 +447,8 @@ __global__ void __launch_bounds__(kThreadsTop, 4)
 #pragma unroll
   for (int i = 0; i < kThreadsTop / 32; ++i) nx += s_n[i];
   // (factors of 1.01: the roundings of the norms and of this expression)
-  const float scale = (float)(H + 64) * 0x1p-24f * 1.01f * sqrtf(nx) * 1.01f;
+  const float under = (float)H * 0x1p-149f;
+  const float scale = (float)(H + 64) * 0x1p-24f * 1.01f * sqrtf(nx + under) * 1.01f;
   for (int e0 = 0; e0 < E; e0 += per) {  // block-uniform
     const int e = e0 + tid % per;
     float a = 0.f, w2 = 0.f;
@@ -475,7 +478,7 @@ __global__ void __launch_bounds__(kThreadsTop, 4)
         w2 += s_p[1][tid + i * per];
       }
       const float b = bias ? bias[(size_t)t * E + e] : 0.f;
-      const float B = scale * sqrtf(w2) + 0x1p-21f * (fabsf(a) + fabsf(b)) + (float)H * 0x1p-148f;
+      const float B = scale * sqrtf(w2 + under) + 0x1p-21f * (fabsf(a) + fabsf(b)) + (float)H * 0x1p-148f;
       s_a[e] = (a + b) - B;
       s_b[e] = (a + b) + B;
       if (!(fabsf(s_b[e]) < INFINITY)) s_all = 1;

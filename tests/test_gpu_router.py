@@ -173,3 +173,28 @@ def test_logits_that_are_not_numbers_rank_last(T, E, k, n_nan):
                 assert np.array_equal(idx[t], oidx) and np.abs(w[t] - og).max() <= G_ATOL, t
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("x_exp,w_exp", [(0, 0), (-80, 0), (0, -75), (-66, -10), (-80, -8), (60, 40)])
+def test_tiled_router_orders_cancelling_logits_at_any_scale(x_exp, w_exp):
+    """Rows of W_r a few units in the last place apart, x nearly orthogonal to them all, both scaled by
+    powers of two (exact): the squares of such values underflow at the small scales, the logits do not,
+    and their order is the oracle's at every scale."""
+    H, E, k, T = 1024, 40, 5, 48
+    shape = Shape(1, H, E, k, 64, synth.Q8_0, model_seed=13)
+    ctx = Ctx(shape, slots=E, max_tokens=T)
+    try:
+        rng = np.random.default_rng(3)
+        w = np.tile(ctx.wr_host[0][:1], (E, 1))
+        for e in range(1, E):
+            at = rng.integers(0, H, 3)
+            w[e, at] = (w[e, at].view(np.int32) + rng.integers(-4, 5, 3).astype(np.int32)).view(np.float32)
+        x = synth.activations(26, 0, 0, 0, T, H).astype(np.float64)
+        w0 = w[0].astype(np.float64)
+        x = (x - np.outer(x @ w0, w0) / (w0 @ w0)).astype(np.float32)
+        w = np.ldexp(w, w_exp)
+        ctx.wr_host[0] = w
+        ctx.wr[0] = ctx.torch.from_numpy(w).to(ctx.device)
+        _check_routes(ctx, np.ldexp(x, x_exp), None, T, k)
+    finally:
+        ctx.close()
