@@ -198,3 +198,28 @@ def test_tiled_router_orders_cancelling_logits_at_any_scale(x_exp, w_exp):
         _check_routes(ctx, np.ldexp(x, x_exp), None, T, k)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("E,k,T", [(8, 8, 16), (40, 5, 33), (128, 8, 65)])
+def test_tiled_router_zero_tokens_and_masked_experts(E, k, T):
+    """Tokens that are all zero (padding) have their biases as logits, and experts masked by a bias of
+    -infinity rank behind all others, the lower first: with and without a bias, beside ordinary tokens."""
+    H = 256
+    shape = Shape(1, H, E, k, 64, synth.Q8_0, model_seed=14)
+    ctx = Ctx(shape, slots=E, max_tokens=T)
+    try:
+        x = synth.activations(27, 0, 0, 0, T, H)
+        x[::3] = 0.0
+        x[3::6] = -0.0
+        idx = _check_routes(ctx, x, None, T, k)
+        assert (idx[::3] == np.arange(k)).all()
+        rng = np.random.default_rng(4)
+        bias = rng.integers(-2, 3, (T, E)).astype(np.float32)  # ties
+        _check_routes(ctx, x, bias, T, k)
+        bias[:, rng.permutation(E)[:E - k]] = -np.inf  # k left
+        _check_routes(ctx, x, bias, T, k)
+        if E > k:  # fewer than k left: the masked experts of the lowest index follow, with weight 0
+            bias[:, np.flatnonzero(bias[0] > -np.inf)[:2]] = -np.inf
+            _check_routes(ctx, x, bias, T, k)
+    finally:
+        ctx.close()
