@@ -95,6 +95,7 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
 __device__ __forceinline__ uint32_t idesc_n(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
 }
+constexpr uint32_t kNegateA = 1u << 13;  // the descriptor's bit that negates A
 // the MMA width of a block with n assignments: n rounded up to a multiple of 16
 __device__ __forceinline__ int n_eff(int n) { return max(16, (n + 15) & ~15); }
 
@@ -111,16 +112,16 @@ __device__ __forceinline__ uint32_t elect_one() {
   return r;
 }
 // the six MMAs of one M block and K step of 32: (hi + lo) B's hi and hi times B's lo, two K = 16 halves (of B two
-// core matrices, of A 8 columns)
+// core matrices, of A 8 columns); A's low part is stored negated (split_pair)
 __device__ __forceinline__ void mma_step(uint32_t d_tmem, uint32_t a, uint64_t bh, uint64_t bl, uint32_t idesc,
                                          uint32_t accumulate) {
   constexpr uint64_t ko = 256 >> 4;
   mma_bf16(d_tmem, a, bh, idesc, accumulate);
   mma_bf16(d_tmem, a, bl, idesc, 1);
-  mma_bf16(d_tmem, a + 16, bh, idesc, 1);
+  mma_bf16(d_tmem, a + 16, bh, idesc | kNegateA, 1);
   mma_bf16(d_tmem, a + 8, bh + ko, idesc, 1);
   mma_bf16(d_tmem, a + 8, bl + ko, idesc, 1);
-  mma_bf16(d_tmem, a + 24, bh + ko, idesc, 1);
+  mma_bf16(d_tmem, a + 24, bh + ko, idesc | kNegateA, 1);
 }
 // arrive on the barrier once every MMA this thread issued so far has completed
 __device__ __forceinline__ void mma_commit_at(uint32_t bar) {
@@ -166,32 +167,58 @@ __device__ __forceinline__ void split2(uint64_t w, uint32_t& hi, uint32_t& lo) {
   lo = bf2_bits(__floats2bfloat162_rn(__uint_as_float(ra), __uint_as_float(rb)));
 }
 
-// A pair of codes q (exact bf16) times the scale d = dh + dl (both bf16, exact: 11 bits) -> the bf16 parts
-// hi = RN(q d), lo = RN(q d - hi) of the weights, in four packed instructions of the FMA pipe: q dh - hi is
-// exact (it fits 8 bits), so each part is rounded once (hi to within 2^-9 of its last place of that for
-// Q8_0, whose q dl is rounded first; hi + lo is as close to q d as before, 1.2e-6 of it in the mean square).
-// Converting q d to fp32 and splitting it there kept the ALU pipe busy with byte permutes and unpacking.
-__device__ __forceinline__ void split_pair(uint32_t q, uint32_t dh, uint32_t dl, uint32_t& hi, uint32_t& lo) {
-  asm("{ .reg .b32 t, n, e;\n"
-      "mul.rn.bf16x2 t, %2, %4;\n"
-      "fma.rn.bf16x2 %0, %2, %3, t;\n"
-      "neg.bf16x2 n, %0;\n"
-      "fma.rn.bf16x2 e, %2, %3, n;\n"
-      "fma.rn.bf16x2 %1, %2, %4, e; }"
-      : "=&r"(hi), "=r"(lo)
-      : "r"(q), "r"(dh), "r"(dl));
+// A scale d as the sum of two bf16 values dh + dl (exact: 11 bits; dl at most four units of d's last place).
+struct ScaleParts {
+  uint32_t h, nh, l, nl, l2;  // pairs of dh, -dh, dl, -dl, 2 dl
+  __device__ __forceinline__ explicit ScaleParts(float d) {
+    const __nv_bfloat16 hb = __float2bfloat16_rn(d), lb = __float2bfloat16_rn(d - __bfloat162float(hb));
+    h = __bfloat16_as_ushort(hb) * 0x10001u;
+    l = __bfloat16_as_ushort(lb) * 0x10001u;
+    nh = h ^ 0x80008000u;
+    nl = l ^ 0x80008000u;
+    l2 = __bfloat16_as_ushort(lb + lb) * 0x10001u;
+  }
+};
+
+// A pair of codes q (exact bf16) times a scale -> the bf16 parts hi = RN(q d) of the weights and -lo, lo =
+// RN(q d - hi), in packed instructions of the FMA pipe: hi - q dh is exact (it fits 8 bits), so each part is
+// rounded once.  (-lo: a sign change in between would cost an instruction; the MMA negates it.)  t = q dl is
+// exact for Q4_0.  For Q8_0 it may take nine bits and is then rounded by one unit, to a multiple of four units:
+// where that makes q dh + t a tie between two values of hi, hi could be the farther one (for ten pairs of code
+// and mantissa hi + lo was off by up to 9.2e-6 of q d, in place of 7.6e-6).  2 q dl - t is off by one unit to the other
+// side, no multiple of four, and meets no tie: hi is the nearest for every code and mantissa.
+// Converting q d to fp32 and splitting it there kept the ALU pipe busy with byte permutes and unpacking: 1000
+// tokens over 64 Q8_0 experts take 324 us a call, so 338 (with the split in f32x2 arithmetic 340; with hi from
+// q dh + RN(q dl), 318).
+template <int QT>
+__device__ __forceinline__ void split_pair(uint32_t q, const ScaleParts& d, uint32_t& hi, uint32_t& nlo) {
+  uint32_t t;
+  if constexpr (QT == MF_Q8_0)
+    asm("{ .reg .b32 m;\n"
+        "mul.rn.bf16x2 m, %1, %2;\n"
+        "fma.rn.bf16x2 %0, %1, %3, m; }"
+        : "=r"(t)
+        : "r"(q), "r"(d.nl), "r"(d.l2));
+  else
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(t) : "r"(q), "r"(d.l));
+  asm("{ .reg .b32 e;\n"
+      "fma.rn.bf16x2 %0, %2, %3, %6;\n"
+      "fma.rn.bf16x2 e, %2, %4, %0;\n"
+      "fma.rn.bf16x2 %1, %2, %5, e; }"
+      : "=&r"(hi), "=r"(nlo)
+      : "r"(q), "r"(d.h), "r"(d.nh), "r"(d.nl), "r"(t));
 }
 
-// Four codes (Q8_0: bytes q + 128; Q4_0: nibbles masked to bytes) -> two words of hi and of lo.
+// Four codes (Q8_0: bytes q + 128; Q4_0: nibbles masked to bytes) -> two words of hi and of -lo.
 template <int QT>
-__device__ __forceinline__ void dequant4(uint32_t w, uint32_t dh, uint32_t dl, uint32_t* h, uint32_t* l) {
+__device__ __forceinline__ void dequant4(uint32_t w, const ScaleParts& d, uint32_t* h, uint32_t* l) {
   uint32_t q01, q23;
   if constexpr (QT == MF_Q8_0)
     dq::codes_q8(w, q01, q23);
   else
     dq::codes_q4(w, q01, q23);
-  split_pair(q01, dh, dl, h[0], l[0]);
-  split_pair(q23, dh, dl, h[1], l[1]);
+  split_pair<QT>(q01, d, h[0], l[0]);
+  split_pair<QT>(q23, d, h[1], l[1]);
 }
 
 // 8 consecutive columns of this thread's TMEM lane
@@ -366,8 +393,7 @@ __global__ void __launch_bounds__(1024, 1)
       const int q = (kk >> 1) & 3;
       const uint32_t sw = q == 0 ? sv.x : q == 1 ? sv.y : q == 2 ? sv.z : sv.w;
       const float dsc = __half2float(__ushort_as_half((unsigned short)((kk & 1) ? (sw >> 16) : (sw & 0xFFFFu))));
-      const __nv_bfloat16 dhb = __float2bfloat16_rn(dsc), dlb = __float2bfloat16_rn(dsc - __bfloat162float(dhb));
-      const uint32_t dh = __bfloat16_as_ushort(dhb) * 0x10001u, dl = __bfloat16_as_ushort(dlb) * 0x10001u;
+      const ScaleParts ds(dsc);
       // 16 weights at a time (elements 0-15, 16-31: the two K halves of the step)
       uint32_t w[8];
       if constexpr (QT == MF_Q8_0) {
@@ -385,7 +411,7 @@ __global__ void __launch_bounds__(1024, 1)
       for (int half = 0; half < 2; ++half) {
         uint32_t h[8], l[8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) dequant4<QT>(w[4 * half + i], dh, dl, h + 2 * i, l + 2 * i);
+        for (int i = 0; i < 4; ++i) dequant4<QT>(w[4 * half + i], ds, h + 2 * i, l + 2 * i);
         if (half == 0) {  // the MMAs have read the stage
           if (s >= kStages) {
             if (!wait(&done[before], bph, 2u)) {

@@ -182,3 +182,50 @@ def test_threshold_arguments():
             mf.mf_prefill_threshold(odd.h, 2)
     finally:
         odd.close()
+
+
+def _rows(bytes_, rows, cols):
+    """Q8_0 tensor bytes [rows x cols] -> (codes int8 [rows, cols / 32, 32], scales binary16 [rows, cols / 32]), views."""
+    b = bytes_.reshape(rows, cols // 32, 34)
+    return b[..., 2:].view(np.int8), b[..., :2].view(np.float16)[..., 0]
+
+
+def test_gemm_weights_keep_sixteen_bits():
+    """Every Q8_0 code of 86 and more with every binary16 mantissa whose product with it takes more than
+    eight bits below the first eight: the two bf16 parts of a weight are the nearest ones, so their sum is
+    within 2^-17 of it.  One hidden feature is exactly 1 (silu(32) 2^-5) and the others 0, so an output is
+    one weight of the down projection, summed with zeros."""
+    E, H, I, T = 6, 4096, 128, 12
+    q = np.arange(87, 128, 2)
+    m = np.arange(1024, 2048)
+    m = m[(m % 8 == 3) | (m % 8 == 5)]
+    qq, mm = [v.reshape(-1) for v in np.meshgrid(q, m)]
+    qq, mm = np.concatenate([qq, -qq]), np.concatenate([mm, mm])  # 10752 pairs
+    qq, mm = np.resize(qq, E * H), np.resize(mm, E * H)
+
+    def edit(layer, e, p):
+        p = np.zeros_like(p)
+        tb = I * H // 32 * 34
+        for at, code, d in ((0, 32, 1.0), (tb, 1, 2.0 ** -5)):
+            c, s = _rows(p[at:at + tb], I, H)
+            c[0, 0, 0], s[0, 0] = code, d
+        c, s = _rows(p[2 * tb:], H, I)
+        c[:, 0, 0] = qq[e * H:(e + 1) * H]
+        s[:, 0] = mm[e * H:(e + 1) * H] / 1024.0
+        return p
+
+    shape = Shape(1, H, E, 1, I, synth.Q8_0, model_seed=15)
+    ctx = Ctx(shape, E, max_tokens=T, edit=edit)
+    try:
+        ctx.mf.mf_prefill_threshold(ctx.h, 2)
+        x = np.zeros((T, H), np.float32)
+        x[:, 0] = 1.0
+        bias = synth.plant_bias((np.arange(T) % E).astype(np.int32)[:, None], E)
+        y, idx, _ = ctx.forward(0, x, bias, T)
+        assert np.array_equal(idx[:, 0], np.arange(T) % E)
+        want = (qq * mm / 1024.0).reshape(E, H)
+        for t in range(T):
+            rel = np.abs(y[t].astype(np.float64) - want[t % E]) / np.abs(want[t % E])
+            assert rel.max() <= 2.0 ** -17, (t, rel.max())
+    finally:
+        ctx.close()
