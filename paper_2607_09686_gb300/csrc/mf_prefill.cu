@@ -188,8 +188,8 @@ struct ScaleParts {
 // and mantissa hi + lo was off by up to 9.2e-6 of q d, in place of 7.6e-6).  2 q dl - t is off by one unit to the other
 // side, no multiple of four, and meets no tie: hi is the nearest for every code and mantissa.
 // Converting q d to fp32 and splitting it there kept the ALU pipe busy with byte permutes and unpacking: 1000
-// tokens over 64 Q8_0 experts take 324 us a call, so 338 (with the split in f32x2 arithmetic 340; with hi from
-// q dh + RN(q dl), 318).
+// tokens over 64 Q8_0 experts took 324 us a call, so 338 (with the split in f32x2 arithmetic 340; with hi from
+// q dh + RN(q dl), 318), each before the epilogue's division was exact (329 us).
 template <int QT>
 __device__ __forceinline__ void split_pair(uint32_t q, const ScaleParts& d, uint32_t& hi, uint32_t& nlo) {
   uint32_t t;
@@ -558,13 +558,14 @@ __global__ void __launch_bounds__(1024, 1)
         // h tile of K step r / 32 of the down GEMM: this lane's row is its k = r % 32
         uint8_t* ht = d.ht + ((size_t)(d.tb_off[un.u] + un.tb) * (d.I / kBK) + (r >> 5)) * kBTile;
         for (int c0 = ch * 64; c0 < min(ne, ch * 64 + 64); c0 += 16) {  // the columns the down MMAs read
+          // (the division is the IEEE one: __fdividef is 0 above 2^126, for gates below -87.3; 1000 tokens 324 -> 329 us)
           float g[16], u[16];
           tmem_ld16(lane_addr + c0, g);
           tmem_ld16(lane_addr + kBN + c0, u);
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             const int col = c0 + q;
-            const float hv = col < n ? __fdividef(g[q], 1.0f + expf(-g[q])) * u[q] : 0.0f;
+            const float hv = col < n ? g[q] / (1.0f + expf(-g[q])) * u[q] : 0.0f;
             const __nv_bfloat16 hi = __float2bfloat16_rn(hv);
             const uint32_t o = core_off(col, r & 31);
             *reinterpret_cast<uint16_t*>(ht + o) = __bfloat16_as_ushort(hi);

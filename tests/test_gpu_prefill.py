@@ -229,3 +229,37 @@ def test_gemm_weights_keep_sixteen_bits():
             assert rel.max() <= 2.0 ** -17, (t, rel.max())
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("gemm", [True, False])
+def test_silu_of_large_negative_gates(gemm):
+    """Gates of -85 .. -88.7, where 1 + exp(-gate) is above 2^122: silu is small but not zero, in the
+    tensor-core path as in the others."""
+    E, H, I, T = 2, 128, 128, 6
+    gates = np.linspace(1.33, 1.3859, I).astype(np.float16)  # times -64: no bits for the parts to lose (an
+    # error of the gate would be magnified by its size in silu)
+
+    def edit(layer, e, p):
+        p = p.copy()
+        tb = I * H // 32 * 34
+        for at, code, d in ((0, -64, gates), (tb, 127, 1000.0)):
+            c, s = _rows(p[at:at + tb], I, H)
+            c[:, 0, 0], s[:, 0] = code, d
+        return p
+
+    shape = Shape(1, H, E, 1, I, synth.Q8_0, model_seed=16)
+    ctx = Ctx(shape, E, max_tokens=T, edit=edit)
+    pays = Payloads(shape, edit=edit)
+    try:
+        ctx.mf.mf_prefill_threshold(ctx.h, 2 if gemm else 0)
+        x = np.zeros((T, H), np.float32)
+        x[:, 0] = 1.0
+        bias = synth.plant_bias((np.arange(T) % E).astype(np.int32)[:, None], E)
+        y, idx, _ = ctx.forward(0, x, bias, T)
+        yo, _, _ = oracle.layer(pays.for_layer(0, range(E)), synth.Q8_0, H, I, 1, ctx.wr_host[0], bias, x)
+        rel = np.linalg.norm(y.astype(np.float64) - yo, axis=1) / np.linalg.norm(yo.astype(np.float64), axis=1)
+        # h's two bf16 parts and the down weights': 2^-17 each, the dropped product of the low parts 2^-18
+        assert rel.max() <= 2.0 ** -15, rel.max()
+        assert -88.72 < (gates.astype(np.float64) * -64).min() < -88.6
+    finally:
+        ctx.close()
