@@ -309,8 +309,8 @@ int mf_test_hold(mf_ctx_t* ctx, int hold);
  * that must not take cudaMalloc's implicit device synchronisation, or plugins confined to a
  * device-memory budget reserved by their host process — can still compute
  *   y = sum_j g[j] * down_j( silu(gate_j x) * (up_j x) ),   j < model->top_k,
- * from expert weights they already hold, without creating a context.  It runs the kernels of
- * a one-token mf_moe_forward; their intermediate h and index tables live in a file-scope
+ * from expert weights they already hold, without creating a context.  It runs the gate/up and
+ * down kernels of a one-token step in two launches; their intermediate h and index tables live in a file-scope
  * device array of 128 KiB + 256 B, which every GPU that loads this library holds until the
  * process exits.
  *   model    hidden, inter, top_k (<= 8) and qtype are used; top_k * inter must be <= 32768
@@ -331,7 +331,8 @@ int mf_test_hold(mf_ctx_t* ctx, int hold);
  * that device (it reads the array's device address and writes its constant tables): make that
  * first call before any stream capture; host threads that make their first call at the same time
  * take turns.  All calls on a device share the array, so calls whose kernels overlap on the GPU
- * (other streams, other host threads) race on it: serialise them.  Nothing in the array needs
+ * (other streams, other host threads) race on it: serialise them.  They may overlap any other
+ * kernels, mf_moe_forward's among them: none of their blocks waits for another block of its launch.  Nothing in the array needs
  * clearing between calls; h is fully rewritten by each call.  A bounded wait that gives up is
  * reported by mf_expert_ffn_noalloc_check. */
 int mf_expert_ffn_noalloc(const mf_model_t* model, const void* experts, const float* g, const float* x,

@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gateup_pipe(Dev d, int layer, c
     s_base[threadIdx.x] = d.pool + ((size_t)layer * d.S_alloc + d.uslot[threadIdx.x]) * d.lay.stride;
   if (threadIdx.x == 0) s_xmax = kNoExp;
   init_barriers(c, sm);
+  pdl_trigger();  // the down kernel's blocks may start as this one's leave
 
   if (warp == kConsumers) {
     if (lane == 0) {
@@ -247,7 +248,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_gateup_pipe(Dev d, int layer, c
 }
 
 // ---------------------------------------------------------------- down + combine, one token
-// Item i = output rows [i*R, (i+1)*R) of all k experts.
+// Item i = output rows [i*R, (i+1)*R) of all k experts.  A programmatic launch behind k_gateup_pipe (launched
+// plainly: everything before it is complete): a block starts where one of that kernel's has left, and its
+// producer fetches weights, which that kernel does not write, before the consumers wait for its end.  (Eight
+// 2048 x 768 Q8_0 experts: 20.5 -> 16.7 us for both.)
 template <int QT, int VPLD>
 __global__ void __launch_bounds__(kThreads, 1) k_down_pipe(Dev d, int layer, float* __restrict__ y, PipeCfg c) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_down_pipe(Dev d, int layer, flo
       drain(c, sm, mine, d.err, d.wait_ns);
     }
   } else {
+    pdl_wait();  // h is complete
     const int j = warp / R, rho = warp % R;  // one (expert, row) task per warp: k * R <= 16
     const bool active = j < k;
     const XQ<QT>* hq = reinterpret_cast<const XQ<QT>*>(sm.vq);
@@ -958,8 +963,7 @@ cudaError_t down_pipe_q(const Dev& d, int layer, float* y, cudaStream_t s) {
     cudaError_t e =                                                                                       \
         cudaFuncSetAttribute(k_down_pipe<QT, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     if (e != cudaSuccess) return e;                                                                       \
-    k_down_pipe<QT, V><<<grid, kThreads, smem, s>>>(d, layer, y, c);                                      \
-    break;                                                                                                \
+    return launch_pdl(true, k_down_pipe<QT, V>, dim3(grid), dim3(kThreads), smem, s, d, layer, y, c);     \
   }
   switch (vpl_for(d.lay.qrow_d / 16)) {
     case 1: MF_DN(1)
@@ -967,7 +971,6 @@ cudaError_t down_pipe_q(const Dev& d, int layer, float* y, cudaStream_t s) {
     default: MF_DN(3)
   }
 #undef MF_DN
-  return cudaGetLastError();
 }
 
 FusedCfg fused_cfg(const Dev& d) {

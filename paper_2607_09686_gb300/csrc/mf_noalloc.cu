@@ -1,10 +1,11 @@
 // mf_expert_ffn_noalloc: the one-token expert FFN for callers that must not allocate.
 //
-// It runs the same kernels as a one-token mf_moe_forward (the fused launch where the shape allows:
-// 14.6 us for eight 2048 x 768 Q8_0 experts against 20.5 us in two launches), but without a context: the
-// weights are the caller's, and the scratch the kernels pass between each other (h, the SwiGLU
-// activations, plus a few small index tables) lives in the file-scope array below instead of in a
-// context's device allocation.
+// It runs the gate/up + SwiGLU and down + combine kernels of a one-token mf_moe_forward in two launches, but
+// without a context: the weights are the caller's, and the scratch the kernels pass between each other (h, the
+// SwiGLU activations, plus a few small index tables) lives in the file-scope array below instead of in a
+// context's device allocation.  Two launches although the fused one is faster (eight 2048 x 768 Q8_0 experts:
+// 16.7 us against 14.6): its blocks wait for each other, so one on every SM must run at the same time, which a
+// context's own fused launch on another stream can prevent.  No block here waits for another block of its launch.
 #include <atomic>
 #include <cstddef>
 #include <cstring>
@@ -21,9 +22,7 @@ struct NoAllocTables {
   int32_t ident[kMaxTopK];        // slot / assignment j of expert j: 0, 1, ..., 7
   int32_t asg_off[kMaxTopK + 1];  // 0, 1, ..., 8
   int32_t info[kMaxTopK][4];      // per top_k: {top_k, 1 wave, 0, 0}
-  int32_t umiss[kMaxTopK];        // no expert is missing
   unsigned err;                   // device error word of the kernels
-  unsigned long long work;        // grid arrival counter of the fused kernel
 };
 
 constexpr size_t kTablesOff = (size_t)kNoAllocMaxH * sizeof(float);
@@ -58,9 +57,7 @@ int setup(int dev) {
     t.info[j][3] = 0;
   }
   t.asg_off[kMaxTopK] = kMaxTopK;
-  for (int j = 0; j < kMaxTopK; ++j) t.umiss[j] = 0;
   t.err = 0;
-  t.work = 0;
   e = cudaMemcpyToSymbol(g_noalloc, &t, sizeof(t), kTablesOff, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return MF_E_CUDA;
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return MF_E_CUDA;  // the tables have landed
@@ -116,15 +113,10 @@ extern "C" int mf_expert_ffn_noalloc(const mf_model_t* model, const void* expert
   d.asg_off = t->asg_off;
   d.info = t->info[m.top_k - 1];
   d.err = &t->err;
-  d.uniq = t->ident;
-  d.umiss = t->umiss;
-  d.work = &t->work;
   d.g = const_cast<float*>(g);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (decode_pipe_ok(d) && ffn_fused_ok(d)) {  // both projections in one launch, as in a one-token call
-    if (launch_ffn_single(d, 0, x, y, s) != cudaSuccess) return MF_E_CUDA;
-  } else if (decode_pipe_ok(d)) {
+  if (decode_pipe_ok(d)) {
     if (launch_gateup_single(d, 0, x, s) != cudaSuccess) return MF_E_CUDA;
     if (launch_down_single_pipe(d, 0, y, s) != cudaSuccess) return MF_E_CUDA;
   } else {

@@ -119,3 +119,48 @@ def test_noalloc_rejects_sizes_beyond_its_scratch():
         with pytest.raises(mf.MFError) as e:
             mf.mf_expert_ffn_noalloc(big, buf, buf, buf, buf)
         assert e.value.status == mf.MF_E_INVAL
+
+
+def _graph_nodes(graph) -> int:
+    import ctypes
+    cuda = ctypes.CDLL("libcuda.so.1")
+    n = ctypes.c_size_t()
+    assert cuda.cuGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
+
+
+def test_noalloc_ffn_beside_another_contexts_calls():
+    """The call is two kernels, gate/up and down, neither of which waits for other blocks of its own launch
+    (the fused launch of a context does), so it may overlap one-token calls on other streams."""
+    import torch
+    import paper_2607_09686_gb300 as mf
+    H, I, k, q = 2048, 768, 8, synth.Q8_0
+    model = mf.Model(1, H, k, k, I, q)
+    pays = [synth.payload(9, 0, e, H, I, q) for e in range(k)]
+    ed = torch.from_numpy(np.concatenate([slot_image(p, H, I, q) for p in pays])).cuda()
+    x = synth.activations(17, 0, 0, 0, 1, H)
+    g = np.full(k, 1.0 / k, np.float32)
+    xd, gd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda(), torch.empty(1, H, device="cuda")
+    mf.mf_expert_ffn_noalloc(model, ed, gd, xd, yd)  # sets the device up
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        mf.mf_expert_ffn_noalloc(model, ed, gd, xd, yd)
+    assert _graph_nodes(graph) == 2
+
+    shape = Shape(1, H, 16, k, I, q, model_seed=5)
+    ctx = Ctx(shape, 16, max_tokens=1)
+    try:
+        y_ref, _, _ = ctx.forward(0, x, None, 1)
+        y2 = torch.empty(1, H, device="cuda")
+        streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+        torch.cuda.synchronize()
+        for _ in range(50):
+            mf.mf_moe_forward(ctx.h, 0, xd, ctx.wr[0], None, 1, y2, stream=streams[0].cuda_stream)
+            mf.mf_expert_ffn_noalloc(model, ed, gd, xd, yd, stream=streams[1].cuda_stream)
+        torch.cuda.synchronize()
+        assert np.array_equal(y2.cpu().numpy(), y_ref)
+        assert_outputs_close(yd.cpu().numpy(), _oracle_ffn(pays, g, x[0], H, I, q))
+        assert mf.mf_check(ctx.h) == mf.MF_OK and mf.mf_expert_ffn_noalloc_check() == mf.MF_OK
+    finally:
+        ctx.close()
