@@ -87,9 +87,27 @@ struct Carve {
 struct ScratchOffsets {
   uint64_t slot_of, expert_of, last_use, clock, stats, tr_n, tr_expert, tr_slot, tr_hit;
   uint64_t zpart, idx, g, uniq, uslot, umiss, asg_off, asg, pos_slot, info, miss_list, h, part;
-  uint64_t work, err, tb_off, sx, sb, sy, sidx, sw, stage, xs, hs, xe, sched;
+  uint64_t work, err, tb_off, sx, sb, sy, sidx, sw, stage, xs, xe, sched;
   uint64_t total;
 };
+
+// the tensor-core path's operand tiles are allocated with the context when max_tokens reaches
+// the default threshold (else on first enabling it)
+bool gemm_at_create(const mf_model_t& m, int Tm) { return Tm >= kPrefillMinTokens && prefill_shape_ok(m.hidden, m.inter); }
+
+// The streaming kernels' activation pieces of a call of Tm tokens: x's, then h's.
+uint64_t stream_x_bytes(const mf_model_t& m, int Tm) { return align256(stream_bytes(Tm, m.hidden)); }
+uint64_t stream_scratch_bytes(const mf_model_t& m, int Tm) {
+  return stream_x_bytes(m, Tm) + stream_bytes(Tm * m.top_k, m.inter);
+}
+
+// Bytes of the tensor-core path's allocation.  Made with the context, it also holds the streaming kernels'
+// pieces: a call takes one path or the other, whatever the threshold is, and calls follow one another.
+uint64_t gemm_alloc_bytes(const mf_model_t& m, int Tm) {
+  const uint64_t tiles = prefill_scratch_bytes(Tm, m.top_k, m.n_experts, m.hidden, m.inter);
+  const uint64_t pieces = gemm_at_create(m, Tm) ? stream_scratch_bytes(m, Tm) : 0;
+  return tiles > pieces ? tiles : pieces;
+}
 
 ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   ScratchOffsets o;
@@ -112,7 +130,7 @@ ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   o.umiss = c.take<int32_t>(E);
   o.asg_off = c.take<int32_t>(E + 1);
   o.asg = c.take<int32_t>((uint64_t)Tm * k);
-  o.pos_slot = c.take<int32_t>((uint64_t)Tm * k);
+  o.pos_slot = c.take<int32_t>(k);
   o.info = c.take<int32_t>(2 + E);
   o.miss_list = c.take<int32_t>(E + S);
   o.h = c.take<float>(k * I);
@@ -128,22 +146,17 @@ ScratchOffsets scratch_layout(const mf_model_t& m, int S, int Tm) {
   o.sw = c.take<float>((uint64_t)Tm * k);
   // calls with several waves stage the next wave's misses: one payload per slot (T_max > 1)
   o.stage = c.take<uint8_t>(Tm > 1 ? (uint64_t)S * make_layout(m).stride : 0);
-  o.xs = c.take<uint8_t>(Tm > 1 ? stream_bytes(Tm, (int)H) : 0);
-  o.hs = c.take<uint8_t>(Tm > 1 ? stream_bytes(Tm * (int)k, (int)I) : 0);
+  const bool pieces = Tm > 1 && !gemm_at_create(m, Tm);  // (else in the tensor-core path's allocation)
+  o.xs = c.take<uint8_t>(pieces ? stream_scratch_bytes(m, Tm) : 0);
   o.xe = c.take<int32_t>(Tm);
   o.total = c.off;
   return o;
 }
 
-// the tensor-core path's operand tiles are allocated with the context when max_tokens reaches
-// the default threshold (else on first enabling it)
-bool gemm_at_create(const mf_model_t& m, int Tm) { return Tm >= kPrefillMinTokens && prefill_shape_ok(m.hidden, m.inter); }
-
 uint64_t overhead_bytes(const mf_model_t& m, int S, int Tm) {
   const Layout lay = make_layout(m);
   const uint64_t padding = (uint64_t)m.n_layers * S * (lay.stride - lay.canonical);
-  const uint64_t gemm =
-      gemm_at_create(m, Tm) ? prefill_scratch_bytes(Tm, m.top_k, m.n_experts, m.hidden, m.inter) : 0;
+  const uint64_t gemm = gemm_at_create(m, Tm) ? gemm_alloc_bytes(m, Tm) : 0;
   return scratch_layout(m, S, Tm).total + padding + gemm;
 }
 
@@ -152,12 +165,16 @@ int alloc_gemm_scratch(mf_ctx* c) {
   Dev& d = c->d;
   const uint64_t tiles = prefill_tiles_max(d.T_max, d.k, d.E);
   uint8_t* p = nullptr;
-  cudaError_t e = cudaMalloc((void**)&p, prefill_scratch_bytes(d.T_max, d.k, d.E, d.H, d.I));
+  cudaError_t e = cudaMalloc((void**)&p, gemm_alloc_bytes(c->model, d.T_max));
   if (e != cudaSuccess) {
     cuda_fail(e, "cudaMalloc(GEMM tiles)");
     return MF_E_OOM;
   }
   c->gemm_scratch = p;
+  if (gemm_at_create(c->model, d.T_max)) {
+    d.xs = p;
+    d.hs = p + stream_x_bytes(c->model, d.T_max);
+  }
   d.xt = p;
   d.ht = p + tiles * (uint64_t)128 * d.H * 4;
   return MF_OK;
@@ -377,7 +394,7 @@ int create_ctx(mf_ctx_t** out, const mf_model_t* m, const mf_plan_t* p, int devi
   d.err = reinterpret_cast<unsigned*>(base + so.err);
   d.sched = reinterpret_cast<unsigned*>(base + so.sched);
   d.xs = base + so.xs;
-  d.hs = base + so.hs;
+  d.hs = d.xs + stream_x_bytes(*m, Tm);
   d.xe = reinterpret_cast<int32_t*>(base + so.xe);
   d.tb_off = reinterpret_cast<int32_t*>(base + so.tb_off);
   c->stage_x = reinterpret_cast<float*>(base + so.sx);
@@ -426,12 +443,12 @@ int create_ctx(mf_ctx_t** out, const mf_model_t* m, const mf_plan_t* p, int devi
   }
   c->tmaps_ok = prefill_shape_ok(d.H, d.I) && prefill_tensor_maps(c) == 0;
   c->prefill_min_t = 0;
-  if (c->tmaps_ok && gemm_at_create(*m, Tm)) {
+  if (gemm_at_create(*m, Tm)) {
     if ((rc = alloc_gemm_scratch(c)) != MF_OK) {
       free_ctx(c);
       return rc;
     }
-    c->prefill_min_t = kPrefillMinTokens;
+    if (c->tmaps_ok) c->prefill_min_t = kPrefillMinTokens;
   }
   *out = c;
   return MF_OK;

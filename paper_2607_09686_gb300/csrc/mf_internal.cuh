@@ -69,7 +69,7 @@ struct Dev {
   int32_t* umiss;      // [E]           1 if the access missed
   int32_t* asg_off;    // [E + 1]       assignments of unique expert u: asg[asg_off[u] .. asg_off[u+1])
   int32_t* asg;        // [T_max * k]   assignment = t * k + j
-  int32_t* pos_slot;   // [T_max * k]   slot serving assignment t * k + j
+  int32_t* pos_slot;   // [k]           slot of the j-th choice (T = 1)
   int32_t* info;       // [2 + E]       U, number of waves, misses of wave w at 2 + w
   int32_t* miss_list;  // [E + S_alloc] unique index of miss m of wave w at w * S_active + m
   float* h;            // [k][I]  SwiGLU activations (T = 1)
@@ -278,7 +278,8 @@ struct mf_ctx {
   bool decode_pipe;  // batch-1 calls use the pipelined decode kernels
   bool ffn_fused;    // ... fused into one cooperative launch
   int prefill_min_t;  // calls with T >= this use the tensor-core grouped GEMMs (0 = never)
-  uint8_t* gemm_scratch;  // x and h tiles of the tensor-core path (allocated when first enabled)
+  uint8_t* gemm_scratch;  // x and h tiles of the tensor-core path (allocated when first enabled); made with the
+                          // context, the streaming kernels' pieces (xs, hs) lie here as well
   bool tmaps_ok;
   CUtensorMap ts_gu[2], ts_d[2];  // the same regions for the streaming kernels: [0] boxes of 64 rows' codes
                                   // of 128 weights, [1] boxes of 64 rows' 8 scales

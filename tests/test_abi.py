@@ -67,6 +67,21 @@ def test_plan_matches_oracle(mf, name):
             assert p.footprint_bytes == p.lower_bound_bytes + p.overhead_bytes and p.overhead_bytes > 0
 
 
+@pytest.mark.parametrize("q", [8, 2])
+def test_plan_overhead_per_token(mf, q):
+    """A context of thousands of tokens holds each further token's tiles and outputs (and staging for host
+    buffers), but no second form of its activations for the path of smaller calls."""
+    H, E, k, I = 2048, 128, 8, 768
+    m = mf.Model(48, H, E, k, I, q)
+    a, b = (mf.mf_plan(m, mf.PlanReq(15.0, 1 << 62, 0, 0, T, 0)).overhead_bytes for T in (16384, 32768))
+    token = k * (H + I) * 4 + k * H * 4 + 2 * H * 4 + E * 4 + 5 * k * 4 + 4  # GEMM tiles, outputs, host staging, routes
+    logits = 2 * E * 4  # of the router's K splits: two at most at these sizes
+    assert token * 16384 <= b - a <= (token + logits) * 16384 * 1.001
+    # a small context holds the pieces of its calls: 6 bytes a value
+    a, b = (mf.mf_plan(m, mf.PlanReq(15.0, 1 << 62, 0, 0, T, 0)).overhead_bytes for T in (64, 128))
+    assert b - a >= (H + k * I) * 6 * 64
+
+
 def test_plan_rejects_bad_arguments(mf):
     lib = ctypes.CDLL(mf.LIB_PATH)
     out = mf.Plan()

@@ -68,3 +68,32 @@ def test_tokens_whose_logits_overflow_leave_the_others_alone(E, k, slots, T):
         assert ctx.mf.mf_check(ctx.h) == 0
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("E,k", [(2, 1), (12, 4)])
+def test_calls_of_both_paths_take_turns(E, k):
+    """A context of 256 tokens and more keeps the streaming kernels' pieces and the GEMMs' tiles in one
+    allocation: calls of both paths, back to back and at every threshold, give the oracle's outputs.  (With two
+    experts and top-1 the pieces are the larger.)"""
+    H, I, T = 256, 128, 1200
+    shape = Shape(1, H, E, k, I, synth.Q8_0, model_seed=17)
+    ctx = Ctx(shape, E, max_tokens=T)
+    pays = Payloads(shape)
+    try:
+        x = synth.activations(41, 0, 0, 0, T, H)
+        yo, io, _ = oracle.layer(pays.for_layer(0, range(E)), synth.Q8_0, H, I, k, ctx.wr_host[0], None, x)
+        torch = ctx.torch
+        xd = torch.from_numpy(x).to(ctx.device)
+        for threshold in (None, 0, 2, 700, 256):
+            if threshold is not None:
+                ctx.mf.mf_prefill_threshold(ctx.h, threshold)
+            sizes = (T, 255, 256, 3, T, 17, 600)
+            ys = [torch.full((n, H), float("nan"), device=ctx.device) for n in sizes]
+            for n, y in zip(sizes, ys):
+                ctx.mf.mf_moe_forward(ctx.h, 0, xd[:n], ctx.wr[0], None, n, y)
+            torch.cuda.synchronize()
+            for n, y in zip(sizes, ys):
+                assert_outputs_close(y.cpu().numpy(), yo[:n], f"threshold {threshold}, T {n}")
+        assert ctx.mf.mf_check(ctx.h) == 0
+    finally:
+        ctx.close()
