@@ -212,7 +212,10 @@ int mf_load_pack(mf_ctx_t** out, const mf_model_t* model, const mf_plan_t* plan,
  * layer must be issued in token order.  Within a call the accesses are the distinct
  * experts of the T tokens in (token, rank) first-occurrence order; when there are more
  * than S of them they are processed in waves of S.  0 <= T <= plan max_tokens; T = 0
- * does nothing.  Inputs must be finite.  Returns after enqueueing (no host sync). */
+ * does nothing.  Inputs must be finite.  Returns after enqueueing (no host sync).
+ * A call with T = 1 may run as one launch whose blocks, one on every SM, wait for each other
+ * (with the limit of mf_wait_limit): one-token calls of different contexts must not overlap on
+ * the GPU, as each could hold SMs that the other needs.  Order them on one stream or by events. */
 int mf_moe_forward(mf_ctx_t* ctx, int layer, const float* x, const float* router_w,
                    const float* logit_bias, int T, float* y, int32_t* idx_out, float* w_out,
                    void* stream);
