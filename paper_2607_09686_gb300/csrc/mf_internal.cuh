@@ -170,7 +170,8 @@ __device__ __forceinline__ bool counter_wait(const unsigned long long* cnt, unsi
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // A launch whose blocks may be scheduled while the stream's previous kernel ends (every kernel launched
-// this way calls pdl_wait before it touches global memory); a plain launch where that is refused or not
+// this way calls pdl_wait before it touches global memory; k_down_pipe's producer may fetch weights earlier, which
+// were complete before the kernel it follows began); a plain launch where that is refused or not
 // asked for (overlap false: after an event wait the predecessor is not a kernel of this stream).
 template <class... P, class... A>
 cudaError_t launch_pdl(bool overlap, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
