@@ -39,7 +39,7 @@
 // Tensor memory: 256 columns of accumulators, 4 A stages of 64 columns.  What bounds it: the MMAs
 // (three products per weight: 768 cycles of a step's 1200 at 128 assignments) and, between two units, the
 // epilogue's reading of the one accumulator set there is room for (150-280 cycles a step).  4096 tokens,
-// 128 Q4_0 experts of 2048 x 768: gate/up 444 us and down 293 us, where units of 128 rows with A in shared
+// 128 Q4_0 experts of 2048 x 768: gate/up 456 us and down 294 us, where units of 128 rows with A in shared
 // memory took 638 and 446.  With A in shared memory the MMAs' operand reads, the converters'
 // stores and the B copies together filled the shared-memory pipe (an M = 128, N = 128, K = 16 MMA
 // reads 8 KiB of it per 64 tensor cycles; down units of 128 rows also loaded a B tile per 128 rows).
